@@ -126,7 +126,8 @@ def stage_work(N, D, npass, ncanon):
 
 
 # The translation units the Algorithm-6 kernels of the ncu records are compiled from.
-KERNEL_SOURCES = ("ve_bound.cu", "ve_df64.cuh", "ve_device.cuh", "ve_fft.cu", "ve_sweep.cu")
+KERNEL_SOURCES = ("ve_bound.cu", "ve_df64.cuh", "ve_device.cuh", "ve_fft.cu", "ve_fx16.cuh",
+                  "ve_sweep.cu")
 
 
 def source_digest(files=KERNEL_SOURCES):
@@ -759,7 +760,7 @@ def general_oracle_rate(name, seconds):
 def general_rate(ve, synth, name, warmup, steps, stream, flush):
     """Sweeps per second of the general solver on workload `name` (CUDA events on the handle's
     stream around each ve_general_iterate(1), L2 flushed before each), then a profiled pass:
-    per-stage times, the X step's Jacobi sweeps, and the roofline of its round kernel."""
+    per-stage times, the X step's passes, and the roofline of its product kernel."""
     import torch
     terms, L = synth.general_terms(name)
     h = general_create(ve, terms, L, ve.ve_default_options(stream=stream.cuda_stream))
@@ -796,23 +797,29 @@ def general_rate(ve, synth, name, warmup, steps, stream, flush):
     stages = {s: {"ms_per_sweep": pms[i] / k_prof, "launches_per_sweep": pl[i] / k_prof,
                   "share": pms[i] / max(1e-12, total)} for i, s in enumerate(ve.GENERAL_STAGES)}
     ms_round = rms / max(1, rounds)
-    flops_round = 10.0 * n * n
+    flops_round = 26.0 * n * n * (n + 16)
     achieved = flops_round / (ms_round * 1e-3) / 1e12
     xstep_ms = (pms[2] + pms[3]) / k_prof
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as fh:
+            tensor_peak = float(json.load(fh)["bf16_tflops"])
+        tensor_source = "MEASURED_PEAKS.json bf16_tflops (of measured)"
+    except (OSError, ValueError, KeyError):
+        tensor_peak, tensor_source = 1900.0, "of fallback"
     return {
         "value": steps / (ms * 1e-3), "ms_per_step": ms / steps,
         "nspins": terms.get("nspins", terms.get("nsites")),
         "clusters": N, "pair_dim": D, "pairs": K, "x_dim": n,
         "launches_per_sweep": sum(pl) / k_prof, "stages": stages,
-        "jacobi_sweeps_per_x_step": jac, "x_steps_first_order": first_order / k_prof,
-        "roofline": {"bound": "alu", "kernel": "k_dense_round", "achieved": achieved,
-                     "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": achieved / FP64_PEAK_TFLOPS,
-                     "peak_source": "nominal FP64 rate of the part (recipe table), not in "
-                                    "MEASURED_PEAKS.json",
+        "passes_per_x_step": jac,
+        "roofline": {"bound": "tensor", "kernel": "k_fx_product", "achieved": achieved,
+                     "peak": tensor_peak, "unit": "TFLOP/s", "frac": achieved / tensor_peak,
+                     "peak_source": tensor_source,
                      "ms_per_launch": ms_round, "traffic": None,
-                     "algorithmic_per_launch": {"flops": flops_round, "bytes": 64.0 * n * n,
-                                                "note": "10 n^2 flops; 8 n^2 words read+written, "
-                                                        "L2-resident"}},
+                     "algorithmic_per_launch": {"flops": flops_round, "bytes": 36.0 * n * n,
+                                                "note": "26 float16 digit products of the upper half "
+                                                        "of an n x n product; three digit matrices "
+                                                        "of 12 bytes an entry, L2-resident"}},
         "x_step_nominal_tflops": 13.0 / 3.0 * n ** 3 / (xstep_ms * 1e-3) / 1e12,
         "last_status": {"iter": st.iter, "energy_per_spin": st.energy_per_spin,
                         "feas_err": st.feas_err, "bound_per_spin": cert.bound_per_spin},
@@ -866,8 +873,7 @@ def run_general(args):
                 "how": "per step: ve_general_set_state from pinned host, ve_general_iterate(1 sweep) "
                        "with status read-back, ve_general_get_state to pinned host; wall clock"},
         "gpu_launches": int(round(g["launches_per_sweep"] * steps)), "roofline": g["roofline"],
-        "stages": g["stages"], "jacobi_sweeps_per_x_step": g["jacobi_sweeps_per_x_step"],
-        "x_steps_first_order": g["x_steps_first_order"],
+        "stages": g["stages"], "passes_per_x_step": g["passes_per_x_step"],
         "x_step_nominal_tflops": g["x_step_nominal_tflops"], "clocks": ck,
         "last_status": g["last_status"],
         "cpu_baseline": {"value": rate, "unit": UNIT, "cores": cores, "kind": "oracle",

@@ -335,8 +335,8 @@ int ve_selftest_bounded_wait(double* seconds);
  * No translation invariance: random fields, inhomogeneous or long-range couplings.  Every
  * cluster i has its own H_i and rho_i, every pair i < j its own H_ij, rho~_ij, Lambda_ij,
  * Lambda1_ij, Lambda2_ij, and X is one dense (N D) x (N D) matrix whose projection X <-
- * Pi_{>=0}(X - eps G) runs as one eigensolve spread over the whole GPU (cyclic Jacobi in the
- * circle ordering, one launch per round, warm-started from the previous sweep's eigenvectors).
+ * Pi_{>=0}(X - eps G) runs over the whole GPU as (Y + sign(Y) Y) / 2, Y = X - eps G, the matrix
+ * sign by a polynomial iteration of float64-accurate products on the tensor cores.
  * The X step takes the ascent sign X - eps G, as ve_create's solver does.
  *
  * The Hamiltonian is a list of terms on nspins spins:
@@ -404,10 +404,8 @@ int ve_general_dims(const ve_general* h, int* N, int* m, int* D, long* K);
  * (sum_i Tr[H_i rho_i] + sum_{i<j} Tr[H_ij rho_ij]) / nspins with the closed-form pair
  * marginals, Eq. (feasErr) as sqrt(sum_{i<j} (|A1 rho_ij - rho_i|^2 + |A2 rho_ij - rho_j|^2 +
  * |rho_ij - rho~_ij|^2) / K), |energy change|, residual = max of the last two.  Synchronous
- * (the X step's eigensolve reads its stopping test on the host once per Jacobi sweep).  The X
- * step starts from the previous sweep's eigenvectors (from V = I on the first sweep and every
- * 256th), and ends either by the exact stopping rule or, once A = V^T Y V is nearly diagonal,
- * with the first-order reconstruction of VE_DENSE_FIRST_ORDER (below), equally accurate.
+ * (the X step reads its convergence test on the host once a pass of the sign iteration: one pass
+ * when no eigenvalue of Y lies within 3e-6 ||Y||_F of zero, at most three).
  * Returns as ve_iterate. */
 int ve_general_iterate(ve_general* h, long max_iter, double tol, ve_status* out);
 int ve_general_get_status(ve_general* h, ve_status* out);
@@ -416,7 +414,8 @@ int ve_general_get_status(ve_general* h, ve_status* out);
  * raw_bound = sum_i lmin(K_i) + sum_{i<j} lmin(K_ij), K_ij = H'_ij + A1^* Lambda1_ij +
  * A2^* Lambda2_ij, K_i = H'_i - sum_{j>i} Lambda1_ij - sum_{j<i} Lambda2_ji; x_min_eig =
  * lmin(X); x_neg_correction = N m max(0, -x_min_eig); bound_per_spin = (raw_bound -
- * x_neg_correction) / nspins.  All in float64 on the GPU.  Synchronous. */
+ * x_neg_correction) / nspins.  All in float64 on the GPU.  The eigensolve of X (cyclic Jacobi over
+ * the whole GPU) starts from the eigenvectors of the handle's last bound.  Synchronous. */
 int ve_general_bound(ve_general* h, ve_cert* out);
 
 /* Packed state: rho_i (N m^2), rho~ (K D^2), Lambda (K D^2), Lambda1 (K m^2), Lambda2 (K m^2),
@@ -428,20 +427,19 @@ int ve_general_get_state(ve_general* h, double* host, size_t bytes);
 int ve_general_set_state(ve_general* h, const double* host, size_t bytes);
 
 /* Per-stage timing with CUDA events around every following sweep: 0 pair pass, 1 cluster
- * marginals + Lambda1/Lambda2 + status, 2 dense eigensolve of the X step (W = Y V, Jacobi
- * sweeps, Rayleigh quotients), 3 reconstruction X = V diag(max(lambda, 0)) V^T.
- * ve_general_profile(h, 1) clears the accumulators; profile_read gives milliseconds and kernel
- * launches per stage (arrays of VE_GENERAL_NSTAGE) and the mean Jacobi sweeps per X step. */
+ * marginals + Lambda1/Lambda2 + status, 2 X step, 3 empty (the X step's last product is part of
+ * stage 2).  ve_general_profile(h, 1) clears the accumulators; profile_read gives milliseconds and
+ * kernel launches per stage (arrays of VE_GENERAL_NSTAGE) and, in *jacobi_sweeps, the mean passes of
+ * the sign iteration per X step. */
 #define VE_GENERAL_NSTAGE 4
 int ve_general_profile(ve_general* h, int enable);
 int ve_general_profile_read(ve_general* h, double* ms, long* launches, double* jacobi_sweeps);
-/* Device time of the profiled X-step Jacobi sweeps alone (CUDA events around each sweep's graph
- * of n - 1 round launches and its convergence test), the round launches they held, and the X
- * steps that ended with the first-order reconstruction (VE_DENSE_FIRST_ORDER below). */
+/* Device time of the profiled X steps and the launches they held (36 products a pass, two launches
+ * before and two after them); *first_order is 0. */
 int ve_general_profile_rounds(ve_general* h, double* ms, long* rounds, long* first_order);
 
-/* Pi_{>=0} of ONE real symmetric n x n matrix (device, row-major; used as (A + A^T)/2) by the
- * whole-GPU eigensolver of the general solver's X step.  n even, 2 <= n <= 1024.  out may alias
+/* Pi_{>=0} of ONE real symmetric n x n matrix (device, row-major; used as (A + A^T)/2) by a
+ * whole-GPU eigensolver (cyclic Jacobi in the circle ordering).  n even, 2 <= n <= 1024.  out may alias
  * in.  workspace: device memory of ve_project_psd_dense_workspace_size(n) bytes (0 for an
  * unsupported n), 256-byte aligned, owned by the caller; it keeps the eigenvectors.
  * flags: VE_DENSE_WARM starts from the eigenvectors left by the previous call on the same
@@ -449,8 +447,7 @@ int ve_general_profile_rounds(ve_general* h, double* ms, long* rounds, long* fir
  * sweep's rotations were small, A = V^T Y V is formed by one GEMM, and when its off-diagonal part
  * E satisfies ||E||_F^4 <= (n u)^2 ||A||_F^2 d^2 and ||E||_F <= d/4 (d = distance of diag(A) from
  * zero, u = 2^-53) the result is V (f(Lambda) + L o E) V^T, f = max(., 0), L the divided
- * differences of f (Daleckii-Krein): as accurate as running the sweeps to the exact rule (the
- * general solver's X step always does this).  Every Jacobi round is one launch over n/2 CTAs;
+ * differences of f (Daleckii-Krein): as accurate as running the sweeps to the exact rule.  Every Jacobi round is one launch over n/2 CTAs;
  * the n - 1 rounds of a sweep are one CUDA graph.  *sweeps (may be NULL) receives the Jacobi
  * sweeps taken, plus 1000 if the first-order reconstruction was used.  Synchronises `stream`
  * (once per Jacobi sweep).  Each call captures and instantiates the graph of a sweep's n - 1

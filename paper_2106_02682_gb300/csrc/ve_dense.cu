@@ -1,6 +1,6 @@
-// ve_dense.cu -- PSD projection of ONE dense real symmetric n x n matrix on the whole GPU: the
-// X step of Algorithm 5 (Khoo & Lindsey, arXiv:2106.02682, Sec. 3.2), X <- Pi_{>=0}(X - eps G),
-// whose (N D) x (N D) matrix has no block structure to batch over.
+// ve_dense.cu -- eigensolve and PSD projection of ONE dense real symmetric n x n matrix on the whole
+// GPU: ve_project_psd_dense, and lmin(X) of the general solver's bound (its X step, which needs no
+// eigenvectors, is in ve_fxsign.cu).
 //
 // Method: cyclic Jacobi in the circle ordering with the matrix kept implicitly as
 // A = V^T Y V, through the eigenvector estimates V (row i of Vt = column v_i) and W = Y V

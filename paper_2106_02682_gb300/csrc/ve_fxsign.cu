@@ -1,0 +1,448 @@
+// ve_fxsign.cu -- the dense X step of Algorithm 5 (Khoo & Lindsey, arXiv:2106.02682, Sec. 3.2),
+// X <- Pi_{>=0}(X - eps G) for one (N D) x (N D) matrix, as Pi(Y) = (Y + sign(Y) Y) / 2 with the
+// matrix sign from a polynomial iteration: nothing but symmetric products, to float64 accuracy, on
+// the tensor cores.
+//
+// Why.  The cyclic Jacobi it replaces is a chain of n - 1 dependent round launches a sweep (7.3 us
+// each at n = 512, 6.8 sweeps warm: 27 ms of a 28 ms sweep), and its work is float64.  Here a
+// projection is 36 products, each one launch that fills the chip.
+//
+// Iteration.  X_0 = Y / ||Y||_F; X <- X (a I + b X^2 + c X^4): ten growth steps with odd quintics
+// (kStep below) that map [l, 1] into [l', 1] with the largest possible l' (found by a linear
+// program; the idea of Chen & Chow 2014's scaled Newton-Schulz iterations), from l = 3e-6 to 0.9841,
+// then two Newton-Schulz steps of order three (15/8, -10/8, 3/8), the first centred on that
+// interval.  The quintics are held to p(x) >= 0.3 x: one that maps a large eigenvalue to a tiny one
+// (the unconstrained optimum sends 1 to l') turns the rounding of the former's eigenvector into a
+// relative error of the latter (the stability condition of Nakatsukasa & Higham 2012).  Eigenvalues
+// below 3e-6 ||Y||_F (rare; measured 1e-5 .. 1e-2 over the general solver's runs) show in
+// ||I - X^2||_F and cost another pass, which starts from the grown X: three passes reach 2.7e-17
+// ||Y||_F, below rounding.  An eigenvalue whose sign has not converged then contributes at most its
+// own size.
+//
+// Products.  As in ve_fx16.cuh (integers as six base-512 float16 digits; planes s + t <= 6, whose
+// error is 2^-56 of max|X| max|Y|), in 16 x 16 blocks stored as the A fragments of mma.sync
+// m16n8k16: a product's output block comes back in that very layout, so each kernel writes the
+// next one's operand digits itself.  32 terms of a plane sum stay below 2^24 (at most 6 x 32 x
+// 256^2), after which the float32 sums go to int64.  All matrices commute and are symmetric: only blocks
+// on and above the diagonal are computed, the others are their transposes (movmatrix).
+// mma.sync rather than tcgen05: the digit planes s + t = q of one output accumulate in registers
+// (seven planes x 128 columns would fill tensor memory with one 128 x 128 tile, and n = 160 .. 512
+// has 2 .. 16 of those for 152 SMs).
+#include "ve_fxsign.h"
+
+#include "ve_fx16.cuh"
+
+namespace ve {
+
+namespace {
+
+using fx16::Frag;
+using fx16::kD;
+
+constexpr int kBlk = kD * 32;   // uint4 of one 16 x 16 block
+constexpr int kWarps = 8;       // warps of a product CTA
+constexpr int kNormCtas = 128;
+constexpr int kSteps = 12;
+constexpr int kMaxPasses = 3;
+constexpr double kResid = 1e-6;  // ||I - X^2||_F^2 before the last step: ||s| - 1| < 3e-10 after it
+
+// x (a + b x^2 + c x^4) of the steps; the eleventh is the order-three Newton-Schulz step on x / m, m
+// the middle of [0.98409, 0.999].  The growth steps stop at 0.999: their slope at 1 is ~10, so a
+// quintic with p(1) = 1 would carry rounding above 1 out of its interval within a few steps.
+struct Step {
+  double a, b, c;
+};
+constexpr double kM = 0.9915432323472013;
+constexpr Step kGrow = {4.0002895, -10.6185218, 7.6172323};
+constexpr Step kStep[kSteps] = {
+    kGrow, kGrow, kGrow, kGrow, kGrow, kGrow, kGrow, kGrow,
+    {3.487584135, -7.220454778, 4.731870643}, {2.352196917, -2.408104863, 1.054907947},
+    {1.875 / kM, -1.25 / (kM * kM * kM), 0.375 / (kM * kM * kM * kM * kM)},
+    {1.875, -1.25, 0.375}};
+
+enum Mode { kSquare, kSquareLast, kPoly, kMul, kFinal };
+
+struct Args {
+  int n, nb;
+  const uint4* A;
+  const uint4* B;
+  uint4* out;
+  long long* y2;
+  long long a, b, c;    // kPoly: a in units of 2^-53, b and c in units of 2^-56
+  double* partial;      // kSquareLast: per-block residuals
+  const FxSignCtl* ctl;
+  const double* Yd;
+  double* Xd;
+  const int* ey;        // kFinal: exponent of Yq's unit
+};
+
+__device__ __forceinline__ uint32_t transpose8(uint32_t v) {
+  uint32_t r;
+  asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(v));
+  return r;
+}
+
+// Digits of the integers z as block (I, J), and transposed as block (J, I).  Of a diagonal block the
+// upper triangle counts: the iteration takes every matrix for exactly symmetric, and would grow an
+// antisymmetric rounding error by its growth factor at every step.
+__device__ __forceinline__ void write_block(const Frag& z, uint4* out, int nb, int I, int J, int lane) {
+  uint32_t d[kD][4];
+  fx16::digits<kD>(z, d);
+  uint4* o = out + ((size_t)I * nb + J) * kBlk + lane;
+  uint4* t = out + ((size_t)J * nb + I) * kBlk + lane;
+  // of a lane's two entries (row, 2 t), (row, 2 t + 1) of an 8 x 8 tile, those below the diagonal
+  const int row = lane >> 2, col = 2 * (lane & 3);
+  const uint32_t below = (col < row ? 0xffffu : 0u) | (col + 1 < row ? 0xffff0000u : 0u);
+#pragma unroll
+  for (int s = 0; s < kD; ++s) {
+    const uint4 v = make_uint4(d[s][0], d[s][1], d[s][2], d[s][3]);
+    const uint4 w = make_uint4(transpose8(v.x), transpose8(v.z), transpose8(v.y), transpose8(v.w));
+    if (I == J) {
+      o[s * 32] = make_uint4((v.x & ~below) | (w.x & below), w.y, v.z, (v.w & ~below) | (w.w & below));
+    } else {
+      o[s * 32] = v;
+      t[s * 32] = w;
+    }
+  }
+}
+
+// x c for |c| < 64 given in units of 2^-56, |x| < 2^55.
+__device__ __forceinline__ long long scale(long long x, long long c) { return __mul64hi(x << 8, c); }
+
+// One product.  A CTA holds TB x TB output blocks of 16 x 16 (blocks TB bi .., TB bj .., bi <= bj),
+// KW warps a block sharing its K range.
+template <int MODE, int TB>
+__global__ void __launch_bounds__(32 * kWarps, 1) k_fx_product(const Args p) {
+  constexpr int KW = kWarps / (TB * TB);
+  __shared__ long long sum[TB * TB][KW > 1 ? KW - 1 : 1][8][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int blk = warp / KW, kw = warp % KW;
+  // tile (bi, bj) of the upper triangle, row by row
+  const int T = (p.nb + TB - 1) / TB;
+  int bi, bj;
+  tri_index(T, blockIdx.x, bi, bj);
+  const int I = bi * TB + blk / TB, J = bj * TB + blk % TB;
+  const bool live = I <= J && J < p.nb;
+  Frag h = {};
+  if (live) {
+    const uint4* a = p.A + (size_t)I * p.nb * kBlk + lane;
+    const uint4* b = p.B + (size_t)J * p.nb * kBlk + lane;
+    const int per = ((p.nb + KW - 1) / KW + 1) & ~1;  // even: the sums are emptied every 2 steps
+    const int k0 = kw * per, k1 = min(p.nb, k0 + per);
+    float acc[2][7][4] = {};
+    uint4 an[kD], bn[kD];
+    if (k0 < k1) {
+#pragma unroll
+      for (int s = 0; s < kD; ++s) {
+        an[s] = a[(size_t)k0 * kBlk + s * 32];
+        bn[s] = b[(size_t)k0 * kBlk + s * 32];
+      }
+    }
+    for (int k = k0; k < k1; ++k) {
+      uint32_t l[kD][4];
+      uint4 r[kD];
+#pragma unroll
+      for (int s = 0; s < kD; ++s) {
+        l[s][0] = an[s].x;
+        l[s][1] = an[s].y;
+        l[s][2] = an[s].z;
+        l[s][3] = an[s].w;
+        r[s] = bn[s];
+      }
+      if (k + 1 < k1) {
+#pragma unroll
+        for (int s = 0; s < kD; ++s) {
+          an[s] = a[(size_t)(k + 1) * kBlk + s * 32];
+          bn[s] = b[(size_t)(k + 1) * kBlk + s * 32];
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < kD; ++t)
+#pragma unroll
+        for (int s = 0; s < kD; ++s)
+          if (s + t <= 6) {
+            fx16::mma(acc[0][s + t], l[s], r[t].x, r[t].z);
+            fx16::mma(acc[1][s + t], l[s], r[t].y, r[t].w);
+          }
+      if (((k - k0) & 1) || k + 1 == k1) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          h[i] += fx16::combine<6>(acc[0], i);
+          h[4 + i] += fx16::combine<6>(acc[1], i);
+        }
+#pragma unroll
+        for (int q = 0; q < 7; ++q)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) acc[0][q][i] = acc[1][q][i] = 0.f;
+      }
+    }
+  }
+  if constexpr (KW > 1) {
+    if (kw > 0) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) sum[blk][kw - 1][i][lane] = h[i];
+    }
+    __syncthreads();
+    if (kw > 0) return;
+#pragma unroll
+    for (int w = 0; w < KW - 1; ++w)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) h[i] += sum[blk][w][i][lane];
+  }
+  if (!live) return;
+  // h: the product in units of 2^50 times the operands' (X, X^2: 2^-53; B: 2^-50)
+  if constexpr (MODE == kSquare || MODE == kSquareLast) {
+    long long* y2 = p.y2 + ((size_t)I * p.nb + J) * 256 + lane;
+    float res = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      h[i] = (h[i] + 4) >> 3;
+      y2[i * 32] = h[i];
+      if constexpr (MODE == kSquareLast) {
+        const int row = fx16::frag_row(i, lane), col = fx16::frag_col(i, lane);
+        const bool diag = I == J && row == col;
+        float e = fx16::unit_float(diag ? (1LL << 53) - h[i] : h[i]);
+        if (diag && 16 * I + row >= p.n) e = 0.f;  // padding
+        res = fmaf(e, e, res);
+      }
+    }
+    write_block(h, p.out, p.nb, I, J, lane);
+    if constexpr (MODE == kSquareLast) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) res += shfl_xor(res, o);
+      if (lane == 0) p.partial[(size_t)I * p.nb + J] = (I == J ? 1.0 : 2.0) * (double)res;
+    }
+  } else if constexpr (MODE == kPoly) {
+    const long long* y2 = p.y2 + ((size_t)I * p.nb + J) * 256 + lane;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      long long v = scale((h[i] + 4) >> 3, p.c) + scale(y2[i * 32], p.b);
+      if (I == J && fx16::frag_row(i, lane) == fx16::frag_col(i, lane)) v += p.a;
+      h[i] = (v + 4) >> 3;  // |B| < 8: units of 2^-50
+    }
+    write_block(h, p.out, p.nb, I, J, lane);
+  } else if constexpr (MODE == kMul) {
+    write_block(h, p.out, p.nb, I, J, lane);
+  } else {
+    const int e = *p.ey - 53 + fx16::product_exp<6>();
+    const bool finite = p.ctl->finite != 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int row = 16 * I + fx16::frag_row(i, lane), col = 16 * J + fx16::frag_col(i, lane);
+      if (row <= col && col < p.n) {
+        const double y = 0.5 * (p.Yd[(size_t)row * p.n + col] + p.Yd[(size_t)col * p.n + row]);
+        const double v = finite ? 0.5 * (y + fx16::word(h[i], e)) : NAN;
+        p.Xd[(size_t)row * p.n + col] = v;
+        p.Xd[(size_t)col * p.n + row] = v;
+      }
+    }
+  }
+}
+
+// Per-CTA sums of squares and largest entries of Y.
+__global__ void __launch_bounds__(256) k_fx_norm(const double* __restrict__ Y, int n, double* partial) {
+  __shared__ double red[8];
+  const size_t nn = (size_t)n * n;
+  double v = 0.0, m = 0.0;
+  for (size_t e = blockIdx.x * (size_t)256 + threadIdx.x; e < nn; e += (size_t)gridDim.x * 256) {
+    v = fma(Y[e], Y[e], v);
+    m = fmax(m, fabs(Y[e]));
+  }
+  v = gsum<256>(v, red);
+  m = -gmin<256>(-m, red);
+  if (threadIdx.x == 0) {
+    partial[blockIdx.x] = v;
+    partial[kNormCtas + blockIdx.x] = m;
+  }
+}
+
+// X_0 = Y / ||Y||_F and Y scaled by its largest entry, as digits; one warp a block on or above the
+// diagonal.  Every warp adds the norms up itself, in one order.
+__global__ void __launch_bounds__(256) k_fx_slice(const double* __restrict__ Y, int n, int nb, const double* partial,
+                                                  uint4* X, uint4* Yq, FxSignCtl* ctl, int* ey) {
+  const int lane = threadIdx.x & 31;
+  double v = 0.0, m = 0.0;
+  for (int k = lane; k < kNormCtas; k += 32) {
+    v += partial[k];
+    m = fmax(m, partial[kNormCtas + k]);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    v += shfl_xor(v, o);
+    m = fmax(m, shfl_xor(m, o));
+  }
+  const bool finite = isfinite(v) != 0;
+  const int E = fx16::exponent_field(m);  // Yq: an entry of the largest one's binade is 2^52 .. 2^53
+  const double inv = finite && v > 0.0 ? (1.0 - 1e-9) * 9007199254740992.0 / sqrt(v) : 0.0;
+  const long w = (long)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (w == 0 && lane == 0) {
+    ctl->fro2 = v;
+    ctl->finite = finite ? 1 : 0;
+    *ey = E - 1075;
+  }
+  if (w >= (long)nb * (nb + 1) / 2) return;
+  int I, J;
+  tri_index(nb, (int)w, I, J);
+  Frag x, q;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int row = 16 * I + fx16::frag_row(i, lane), col = 16 * J + fx16::frag_col(i, lane);
+    double y = 0.0;
+    if (finite && row < n && col < n) y = 0.5 * (Y[(size_t)row * n + col] + Y[(size_t)col * n + row]);
+    x[i] = __double2ll_rn(y * inv);
+    q[i] = fx16::fix(y, E);
+  }
+  write_block(x, X, nb, I, J, lane);
+  write_block(q, Yq, nb, I, J, lane);
+}
+
+// The convergence test: block residuals added in a fixed order.
+__global__ void __launch_bounds__(256) k_fx_check(const double* partial, int nb, FxSignCtl* ctl) {
+  __shared__ double red[8];
+  double v = 0.0;
+  for (int e = threadIdx.x; e < nb * nb; e += 256)
+    if (e / nb <= e % nb) v += partial[e];
+  v = gsum<256>(v, red);
+  if (threadIdx.x == 0) {
+    ctl->resid = v;
+    ctl->done = v <= kResid || ctl->fro2 == 0.0 || !ctl->finite;
+  }
+}
+
+// 32 x 32 tiles where they fill the chip; else one block a CTA with its K range shared by all the
+// warps (n = 160: 55 CTAs instead of 15).
+template <int MODE>
+cudaError_t launch(const Args& a, cudaStream_t s) {
+  const int T = (a.nb + 1) / 2;
+  if (T * (T + 1) / 2 >= 100) {
+    k_fx_product<MODE, 2><<<T * (T + 1) / 2, 32 * kWarps, 0, s>>>(a);
+  } else {
+    k_fx_product<MODE, 1><<<a.nb * (a.nb + 1) / 2, 32 * kWarps, 0, s>>>(a);
+  }
+  return cudaGetLastError();
+}
+
+size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+// One pass from X[0] to X[0] (kSteps is even), the final product and the test.
+cudaError_t issue_pass(FxSignWs& w, const double* Y, double* X, cudaStream_t s) {
+  Args a;
+  a.n = w.n;
+  a.nb = w.nb;
+  a.y2 = w.y2;
+  a.partial = w.partial + 2 * kNormCtas;
+  a.ctl = w.ctl;
+  a.Yd = Y;
+  a.Xd = X;
+  a.ey = reinterpret_cast<const int*>(w.ctl + 1);
+  cudaError_t e = cudaSuccess;
+  for (int k = 0; k < kSteps && e == cudaSuccess; ++k) {
+    a.A = a.B = w.X[k & 1];
+    a.out = w.Y2;
+    e = k == kSteps - 1 ? launch<kSquareLast>(a, s) : launch<kSquare>(a, s);
+    if (e != cudaSuccess) return e;
+    a.A = a.B = w.Y2;
+    a.out = w.B;
+    a.a = (long long)(kStep[k].a * 9007199254740992.0);
+    a.b = (long long)(kStep[k].b * 72057594037927936.0);
+    a.c = (long long)(kStep[k].c * 72057594037927936.0);
+    if ((e = launch<kPoly>(a, s)) != cudaSuccess) return e;
+    a.A = w.X[k & 1];
+    a.B = w.B;
+    a.out = w.X[(k + 1) & 1];
+    e = launch<kMul>(a, s);
+  }
+  if (e != cudaSuccess) return e;
+  a.A = w.X[0];
+  a.B = w.Yq;
+  if ((e = launch<kFinal>(a, s)) != cudaSuccess) return e;
+  k_fx_check<<<1, 256, 0, s>>>(a.partial, w.nb, w.ctl);
+  return cudaGetLastError();
+}
+
+cudaError_t build_graph(FxSignWs& w, const double* Y, double* X, bool first, cudaGraphExec_t* out) {
+  cudaStream_t cs = nullptr;
+  cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
+  if (e != cudaSuccess) return e;
+  e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
+  if (e == cudaSuccess) {
+    if (first) {
+      k_fx_norm<<<kNormCtas, 256, 0, cs>>>(Y, w.n, w.partial);
+      const int blocks = w.nb * (w.nb + 1) / 2;
+      k_fx_slice<<<(blocks + 7) / 8, 256, 0, cs>>>(Y, w.n, w.nb, w.partial, w.X[0], w.Yq, w.ctl,
+                                                   reinterpret_cast<int*>(w.ctl + 1));
+      e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = issue_pass(w, Y, X, cs);
+    cudaGraph_t g = nullptr;
+    const cudaError_t e2 = cudaStreamEndCapture(cs, &g);
+    if (e == cudaSuccess) e = e2;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(out, g, 0);
+    if (g) cudaGraphDestroy(g);
+  }
+  cudaStreamDestroy(cs);
+  return e;
+}
+
+}  // namespace
+
+size_t fxsign_ws_bytes(int n) {
+  if (n < 2 || (n & 1)) return 0;
+  const size_t nb = (n + 15) / 16;
+  return 5 * al256(nb * nb * kBlk * sizeof(uint4)) + al256(nb * nb * 256 * sizeof(long long)) +
+         al256((2 * kNormCtas + nb * nb) * sizeof(double)) + al256(sizeof(FxSignCtl) + sizeof(int));
+}
+
+int fxsign_ws_init(FxSignWs& w, int n, void* mem, size_t bytes) {
+  const size_t need = fxsign_ws_bytes(n);
+  if (need == 0 || !mem || bytes < need || ((uintptr_t)mem & 255)) return -1;
+  w = FxSignWs();
+  w.n = n;
+  w.nb = (n + 15) / 16;
+  unsigned char* p = (unsigned char*)mem;
+  const size_t nb2 = (size_t)w.nb * w.nb;
+  uint4** bufs[5] = {&w.X[0], &w.X[1], &w.Y2, &w.B, &w.Yq};
+  for (auto b : bufs) {
+    *b = (uint4*)p;
+    p += al256(nb2 * kBlk * sizeof(uint4));
+  }
+  w.y2 = (long long*)p;
+  p += al256(nb2 * 256 * sizeof(long long));
+  w.partial = (double*)p;
+  p += al256((2 * kNormCtas + nb2) * sizeof(double));
+  w.ctl = (FxSignCtl*)p;
+  return 0;
+}
+
+void fxsign_ws_release(FxSignWs& w) {
+  if (w.first) cudaGraphExecDestroy(w.first);
+  if (w.again) cudaGraphExecDestroy(w.again);
+  if (w.hctl) cudaFreeHost(w.hctl);
+  w.first = w.again = nullptr;
+  w.hctl = nullptr;
+}
+
+cudaError_t fxsign_project(FxSignWs& w, const double* Y, double* X, cudaStream_t s) {
+  cudaError_t e;
+  if (!w.hctl && (e = cudaMallocHost((void**)&w.hctl, sizeof(FxSignCtl))) != cudaSuccess) return e;
+  if (w.first && (w.Yd != Y || w.Xd != X)) {
+    cudaGraphExecDestroy(w.first);
+    if (w.again) cudaGraphExecDestroy(w.again);
+    w.first = w.again = nullptr;
+  }
+  if (!w.first) {
+    if ((e = build_graph(w, Y, X, true, &w.first)) != cudaSuccess) return e;
+    w.Yd = Y;
+    w.Xd = X;
+  }
+  for (w.passes = 1;; ++w.passes) {
+    if (w.passes > 1 && !w.again && (e = build_graph(w, Y, X, false, &w.again)) != cudaSuccess) return e;
+    if ((e = cudaGraphLaunch(w.passes == 1 ? w.first : w.again, s)) != cudaSuccess) return e;
+    w.launches += 3 * kSteps + 2 + (w.passes == 1 ? 2 : 0);
+    if ((e = cudaMemcpyAsync(w.hctl, w.ctl, sizeof(FxSignCtl), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
+    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
+    if (w.hctl->done || w.passes == kMaxPasses) return cudaSuccess;
+  }
+}
+
+}  // namespace ve

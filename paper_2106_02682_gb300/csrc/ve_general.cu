@@ -29,6 +29,7 @@
 #include "../../include/ve.h"
 #include "ve_dense.h"
 #include "ve_device.cuh"
+#include "ve_fxsign.h"
 #include "ve_internal.h"
 
 namespace ve {
@@ -596,16 +597,17 @@ struct ve_general {
          *parti = nullptr, *Y = nullptr, *vstore = nullptr, *lmin_p = nullptr, *lmin_c = nullptr;
   int *pi = nullptr, *pj = nullptr;
   GenStatus *dst = nullptr, *hst = nullptr;
-  DenseWs dws, bws;  // X-step eigensolver; the bound's eigensolve of X
+  FxSignWs sws;      // the X step (ve_fxsign.cu)
+  DenseWs bws;       // the bound's eigensolve of X
+  long bounds = 0;   // of those so far (each starts from the eigenvectors of the one before)
   bool pair_warm = false;
   int fermionic = 0;
-  long projections = 0;
   // profiling: 0 pair pass, 1 cluster + dual + status, 2 dense eigensolve, 3 reconstruction
   bool prof = false;
   cudaEvent_t ev[VE_GENERAL_NSTAGE + 1] = {};
   double prof_ms[VE_GENERAL_NSTAGE] = {};
   long prof_launch[VE_GENERAL_NSTAGE] = {};
-  long prof_sweeps = 0, prof_solves = 0, prof_dk = 0;
+  long prof_steps = 0, prof_solves = 0;
 };
 
 namespace {
@@ -627,8 +629,8 @@ struct Guard {
   }
 };
 
-// Every refresh-th projection restarts the X eigensolve from V = I, so that rounding in the
-// rotated eigenvectors cannot accumulate over a long run.
+// Every refresh-th bound restarts its eigensolve of X from V = I, so that rounding in the rotated
+// eigenvectors cannot accumulate.
 constexpr long kRefresh = 256;
 
 GenArgs gen_args(ve_general* h) {
@@ -680,14 +682,11 @@ int sweep(ve_general* h) {
   VG_CU(cudaGetLastError());
   h->pair_warm = true;
   stage_mark(h, 2);
-  const long l0 = h->dws.launches;
-  const int mode = (h->projections % kRefresh == 0) ? DENSE_COLD : DENSE_WARM;
-  VG_CU(dense_eig(h->dws, h->Y, mode, s));
-  const long l1 = h->dws.launches;
+  const long l0 = h->sws.launches;
+  VG_CU(fxsign_project(h->sws, h->Y, h->X, s));
+  const long l1 = h->sws.launches;
   stage_mark(h, 3);
-  VG_CU(dense_reconstruct(h->dws, h->X, s));
   stage_mark(h, 4);
-  ++h->projections;
   if (h->prof) {
     VG_CU(cudaEventSynchronize(h->ev[4]));
     for (int k = 0; k < VE_GENERAL_NSTAGE; ++k) {
@@ -698,10 +697,8 @@ int sweep(ve_general* h) {
     h->prof_launch[0] += 1;
     h->prof_launch[1] += 3;
     h->prof_launch[2] += l1 - l0;
-    h->prof_launch[3] += 1;
-    h->prof_sweeps += h->dws.last_sweeps;
+    h->prof_steps += h->sws.passes;
     h->prof_solves += 1;
-    h->prof_dk += h->dws.dk_mode == 2 ? 1 : 0;
   }
   return VE_OK;
 }
@@ -979,11 +976,11 @@ int create_from_blocks(int N, int L, std::vector<double>& Hi, std::vector<double
   }
   h->state_count = (size_t)N * m * m + (size_t)K * (2 * D * D + 2 * m * m) + (size_t)n * n;
   const size_t nd = (size_t)n * n;
-  const size_t dense = dense_ws_bytes((int)n);
+  const size_t dense = dense_ws_bytes((int)n), sign = fxsign_ws_bytes((int)n);
   size_t bytes = al256(h->state_count * 8) + al256(Hi.size() * 8) + al256(Hij.size() * 8) +
                  2 * al256((size_t)K * m * m * 8) + al256((size_t)K * 3 * 8) + al256((size_t)N * 8) +
                  al256(nd * 8) + al256((size_t)K * D * D * 8) + al256((size_t)K * 8) + al256((size_t)N * 8) +
-                 2 * al256((size_t)K * 4) + al256(sizeof(GenStatus)) + 2 * dense;
+                 2 * al256((size_t)K * 4) + al256(sizeof(GenStatus)) + al256(sign) + dense;
   if (cudaMalloc(&h->dev, bytes) != cudaSuccess) {
     delete h;
     return VE_ENOMEM;
@@ -1014,13 +1011,11 @@ int create_from_blocks(int N, int L, std::vector<double>& Hi, std::vector<double
   h->pi = (int*)take((size_t)K * 4);
   h->pj = (int*)take((size_t)K * 4);
   h->dst = (GenStatus*)take(sizeof(GenStatus));
-  void* dmem = take(dense);
+  void* smem = take(sign);
   void* bmem = take(dense);
   int rc = VE_OK;
-  if (dense_ws_init(h->dws, (int)n, dmem, dense) != 0 || dense_ws_init(h->bws, (int)n, bmem, dense) != 0)
+  if (fxsign_ws_init(h->sws, (int)n, smem, sign) != 0 || dense_ws_init(h->bws, (int)n, bmem, dense) != 0)
     rc = VE_EINVAL;
-  // the X step may end with the first-order correction; the bound's eigensolve of X stays exact
-  h->dws.allow_dk = true;
   if (rc == VE_OK) {
     if (o.stream) {
       h->stream = (cudaStream_t)o.stream;
@@ -1064,7 +1059,7 @@ void ve_general_destroy(ve_general* h) {
   if (!h) return;
   Guard g(h->device);
   if (h->stream) cudaStreamSynchronize(h->stream);
-  dense_ws_release(h->dws);
+  fxsign_ws_release(h->sws);
   dense_ws_release(h->bws);
   for (int k = 0; k <= VE_GENERAL_NSTAGE; ++k)
     if (h->ev[k]) cudaEventDestroy(h->ev[k]);
@@ -1129,10 +1124,9 @@ int ve_general_bound(ve_general* h, ve_cert* out) {
   GenArgs a = gen_args(h);
   VG_CU(launch_gbound_pair(a, h->lmin_p, s));
   VG_CU(launch_small(a, 2, h->lmin_c, s));
-  // lmin(X): the eigensolve starts from the X step's eigenvectors (those of Y, which X shares)
-  const size_t nd = (size_t)h->n * h->n * sizeof(double);
-  VG_CU(cudaMemcpyAsync(h->bws.Vt, h->dws.Vt, nd, cudaMemcpyDeviceToDevice, s));
-  VG_CU(dense_eig(h->bws, h->X, h->projections > 0 ? DENSE_WARM : DENSE_COLD, s));
+  // lmin(X): the eigensolve starts from the last bound's eigenvectors
+  VG_CU(dense_eig(h->bws, h->X, h->bounds % kRefresh ? DENSE_WARM : DENSE_COLD, s));
+  ++h->bounds;
   VG_CU(dense_lmin_certified(h->bws, s));
   std::vector<double> lp((size_t)h->K), lc((size_t)h->N);
   DenseCtl ctl;
@@ -1182,14 +1176,11 @@ int ve_general_set_state(ve_general* h, const double* host, size_t bytes) {
 int ve_general_profile(ve_general* h, int enable) {
   if (!h) return VE_EINVAL;
   h->prof = enable != 0;
-  h->dws.prof = h->prof;
-  h->dws.graph_ms = 0.0;
-  h->dws.graph_rounds = 0;
   for (int k = 0; k < VE_GENERAL_NSTAGE; ++k) {
     h->prof_ms[k] = 0.0;
     h->prof_launch[k] = 0;
   }
-  h->prof_sweeps = h->prof_solves = h->prof_dk = 0;
+  h->prof_steps = h->prof_solves = 0;
   return VE_OK;
 }
 
@@ -1199,15 +1190,15 @@ int ve_general_profile_read(ve_general* h, double* ms, long* launches, double* j
     if (ms) ms[k] = h->prof_ms[k];
     if (launches) launches[k] = h->prof_launch[k];
   }
-  if (jacobi_sweeps) *jacobi_sweeps = h->prof_solves ? (double)h->prof_sweeps / h->prof_solves : 0.0;
+  if (jacobi_sweeps) *jacobi_sweeps = h->prof_solves ? (double)h->prof_steps / h->prof_solves : 0.0;
   return VE_OK;
 }
 
 int ve_general_profile_rounds(ve_general* h, double* ms, long* rounds, long* first_order) {
   if (!h) return VE_EINVAL;
-  if (ms) *ms = h->dws.graph_ms;
-  if (rounds) *rounds = h->dws.graph_rounds;
-  if (first_order) *first_order = h->prof_dk;
+  if (ms) *ms = h->prof_ms[2];
+  if (rounds) *rounds = h->prof_launch[2];
+  if (first_order) *first_order = 0;
   return VE_OK;
 }
 
