@@ -50,8 +50,8 @@ extern "C" {
 #define VE_PREC_DF64 2  /* the pair pass and both PSD projections in double-float words (an
                            unevaluated sum of two float32 numbers: 48-bit significand, ~2^-48
                            rounding against float64's 2^-53) on the float32 pipe, everything
-                           else in float64; with 16 x 16 marginals the float64 code is the
-                           faster of the two and runs in this mode as well                    */
+                           else in float64; with 16 x 16 and 64 x 64 marginals the float64
+                           code is the faster of the two and runs in this mode as well        */
 
 #define VE_MAX_BONDS 4
 

@@ -26,6 +26,7 @@
 #include "../../include/ve.h"
 #include "ve_device.cuh"
 #include "ve_fx16.cuh"
+#include "ve_fx64.cuh"
 #include "ve_internal.h"
 
 namespace ve {
@@ -557,6 +558,53 @@ __global__ void __launch_bounds__(32, 16)
   }
 }
 
+// The same for D = 64 in float64 and double-float: one CTA of ten warps per canonical wavevector, the
+// projection by the sign iteration of ve_fx64.cuh (no eigenvectors, so no store).  Unpacked entries
+// are recomputed where the iteration needs them; the result passes through shared memory, where an
+// entry meets the one it shares a packed sequence with.
+// Measured (86 blocks of the 170-cluster chain, one wave): 701 us; 6243 us as float64 Jacobi sweeps.
+__global__ void __launch_bounds__(fx64::kThreads, 1)
+    k_xproj64(double2* spec, const int* __restrict__ canon, const int ncanon, const FftPlan p, const double invN,
+              unsigned long long* stats) {
+  constexpr int D = 64, E = D * D / 2, LD = D + 1;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double* Yr = reinterpret_cast<double*>(smem_raw);  // over the iterate, when that is done with
+  double* Yi = Yr + D * LD;
+  static_assert(2 * sizeof(double) * D * LD <= fx64::Smem<true>::matrix, "layout");
+  const int tid = threadIdx.x;
+  for (int j = blockIdx.x; j < ncanon; j += gridDim.x) {
+    const int s = canon[j], s2 = partner_slot(p, s);
+    double2* z1 = spec + (long)s * E;
+    double2* z2 = spec + (long)s2 * E;
+    auto unpacked = [&](int f, double& re, double& im) {  // 2 C_k
+      const double2 z = z1[f < E ? f : f - E], zz = z2[f < E ? f : f - E];
+      re = f < E ? z.x + zz.x : z.y + zz.y;
+      im = f < E ? z.y - zz.y : zz.x - z.x;
+    };
+    fx64::project<true>(
+        smem_raw, tid,
+        [&](int r, int c, double& re, double& im) {
+          double ar, ai, br, bi;
+          unpacked(r * D + c, ar, ai);
+          unpacked(c * D + r, br, bi);
+          re = 0.25 * (ar + br);
+          im = 0.25 * (ai - bi);
+        },
+        [&](int r, int c, double re, double im) {
+          Yr[r * LD + c] = re;
+          Yi[r * LD + c] = im;
+        });
+    if (stats && tid == 0) atomicAdd(stats + 1, 1ull);
+    for (int e = tid; e < E; e += fx64::kThreads) {
+      const int o1 = (e / D) * LD + e % D, o2 = ((e + E) / D) * LD + e % D;
+      const double y1r = Yr[o1] * invN, y1i = Yi[o1] * invN, y2r = Yr[o2] * invN, y2i = Yi[o2] * invN;
+      z1[e] = make_double2(y1r - y2i, y1i + y2r);
+      if (s2 != s) z2[e] = make_double2(y1r + y2i, y2r - y1i);
+    }
+    __syncthreads();
+  }
+}
+
 // One CTA: canonical slots in increasing order (block-wide scan over chunks of 256 slots).
 __global__ void __launch_bounds__(256) k_canon_list(const FftPlan p, int* canon) {
   __shared__ int scan[256];
@@ -1017,6 +1065,18 @@ cudaError_t launch_xproj16(const FftPlan& p, double2* spec, const int* canon, vo
   return cudaGetLastError();
 }
 
+cudaError_t launch_xproj64(const FftPlan& p, double2* spec, const int* canon, cudaStream_t s,
+                           unsigned long long* stats) {
+  const size_t smem = fx64::Smem<true>::bytes;
+  static unsigned long long mask = 0;
+  cudaError_t e = smem_once(k_xproj64, smem, mask);
+  if (e != cudaSuccess) return e;
+  const int nc = fft_ncanon(p);
+  const long res = resident_grid((const void*)k_xproj64, fx64::kThreads, smem);
+  k_xproj64<<<(unsigned)(nc < res ? nc : res), fx64::kThreads, smem, s>>>(spec, canon, nc, p, 1.0 / p.N, stats);
+  return cudaGetLastError();
+}
+
 template <int D>
 cudaError_t launch_xproj_d(const FftPlan& p, double2* spec, const int* canon, int arith,
                            void* vstore, int warm, cudaStream_t s, unsigned long long* stats,
@@ -1024,6 +1084,8 @@ cudaError_t launch_xproj_d(const FftPlan& p, double2* spec, const int* canon, in
   if (arith == ARITH_FP32) return launch_xproj_t<D, float>(p, spec, canon, vstore, warm, s, stats, gws, iter);
   if constexpr (D == 16) {
     if (arith == ARITH_FP64 || arith == ARITH_DF64) return launch_xproj16(p, spec, canon, vstore, warm, s, stats);
+  } else if constexpr (D == 64) {
+    if (arith == ARITH_FP64 || arith == ARITH_DF64) return launch_xproj64(p, spec, canon, s, stats);
   } else {
     if (arith == ARITH_FP64) return launch_xproj_t<D, double>(p, spec, canon, vstore, warm, s, stats, gws, iter);
     if (arith == ARITH_DF64) return launch_xproj_t<D, df64>(p, spec, canon, vstore, warm, s, stats, gws, iter);

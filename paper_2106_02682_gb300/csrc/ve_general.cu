@@ -29,6 +29,8 @@
 #include "../../include/ve.h"
 #include "ve_dense.h"
 #include "ve_device.cuh"
+#include "ve_fx16.cuh"
+#include "ve_fx64.cuh"
 #include "ve_fxsign.h"
 #include "ve_internal.h"
 
@@ -78,6 +80,11 @@ __host__ __device__ __forceinline__ long pair_index(int N, int i, int j) {
   return (long)i * N - (long)i * (i + 1) / 2 + (j - i - 1);
 }
 
+// The projections of 16 x 16 and 64 x 64 marginals run in fixed point on the tensor cores
+// (ve_fx16.cuh: one warp; ve_fx64.cuh: ten warps), as the translation-invariant solver's do.
+template <int D>
+constexpr int kPairThreads = D == 64 ? fx64::kThreads : GroupShape<D>::NT;
+
 template <int D>
 struct GenSmem {
   static constexpr int m = ClusterDim<D>::m, LD = GroupShape<D>::LD;
@@ -85,9 +92,10 @@ struct GenSmem {
   static constexpr size_t R = 0;                                     // D*D  rhs, then rho
   static constexpr size_t Xs = R + al(sizeof(double) * D * D);       // D*D  X_ij
   static constexpr size_t A = Xs + al(sizeof(double) * D * D);       // D*LD
-  static constexpr size_t V = A + al(sizeof(double) * D * LD);
-  static constexpr size_t WT = V + al(sizeof(double) * D * LD);
-  static constexpr size_t CS = WT + al(sizeof(double) * D * LD);     // D
+  static constexpr size_t V = A + al(sizeof(double) * D * LD);       // D*LD, or the fixed-point forms'
+  static constexpr size_t fx = D == 16 ? fx16::Smem<false>::bytes : D == 64 ? fx64::Smem<false>::bytes : 0;
+  static constexpr size_t WT = V + (fx ? al(fx) : al(sizeof(double) * D * LD));
+  static constexpr size_t CS = WT + (fx ? 0 : al(sizeof(double) * D * LD));  // D
   static constexpr size_t W = CS + al(sizeof(double) * D);           // D
   static constexpr size_t TR = W + al(sizeof(double) * D);           // 2 m^2
   static constexpr size_t RED = TR + al(sizeof(double) * (2 * m * m + 2));
@@ -95,9 +103,9 @@ struct GenSmem {
 };
 
 template <int D>
-__global__ void __launch_bounds__(GroupShape<D>::NT, GroupShape<D>::MINB) k5_pair(const GenArgs a) {
+__global__ void __launch_bounds__(kPairThreads<D>, D == 64 ? 1 : GroupShape<D>::MINB) k5_pair(const GenArgs a) {
   using T = double;
-  constexpr int m = ClusterDim<D>::m, NT = GroupShape<D>::NT, LD = GroupShape<D>::LD;
+  constexpr int m = ClusterDim<D>::m, NT = kPairThreads<D>, LD = GroupShape<D>::LD;
   using S = GenSmem<D>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int tid = threadIdx.x;
@@ -174,8 +182,8 @@ __global__ void __launch_bounds__(GroupShape<D>::NT, GroupShape<D>::MINB) k5_pai
     }
     gsync<NT>();
     T* vs = a.vstore + p * D * D;
-    bool dk = false;
-    if (a.warm) {
+    [[maybe_unused]] bool dk = false;
+    if (D == 4 && a.warm) {
       for (int e = tid; e < D * D; e += NT) V[(e / D) * LD + (e % D)] = vs[e];
     }
     // C = rho - Lambda / mu, symmetrised, into A
@@ -187,65 +195,88 @@ __global__ void __launch_bounds__(GroupShape<D>::NT, GroupShape<D>::MINB) k5_pai
       A[j * LD + i] = v;
     }
     gsync<NT>();
-    if (a.warm) {
-      // A <- V^T C V with the previous eigenvectors
-      for (int e = tid; e < D * D; e += NT) {
-        const int i = e / D, j = e % D;
-        T acc = T(0);
-#pragma unroll 4
-        for (int k = 0; k < D; ++k) acc += A[i * LD + k] * V[k * LD + j];
-        Wt[i * LD + j] = acc;
-      }
-      gsync<NT>();
-      for (int t = tid; t < D * (D + 1) / 2; t += NT) {
-        int i, j;
-        tri_index(D, t, i, j);
-        T acc = T(0);
-#pragma unroll 4
-        for (int k = 0; k < D; ++k) acc += V[k * LD + i] * Wt[k * LD + j];
-        A[i * LD + j] = acc;
-        A[j * LD + i] = acc;
-      }
-      gsync<NT>();
-      jacobi_sym<T, D, LD, NT, true, false, true>(A, V, cs, red, tid, &dk);
-    } else {
-      jacobi_sym<T, D, LD, NT, true, true, true>(A, V, cs, red, tid, &dk);
-    }
-    for (int e = tid; e < D * D; e += NT) vs[e] = V[(e / D) * LD + (e % D)];
-    if (dk) {
-      // first-order (Daleckii-Krein) reconstruction V M V^T, M = f(Lambda) + L o E
-      dk_matrix_sym<T, D, LD, NT>(A, cs, tid);
-      for (int e = tid; e < D * D; e += NT) {
-        const int i = e / D, j = e % D;
-        T acc = T(0);
-#pragma unroll 4
-        for (int k = 0; k < D; ++k) acc += V[i * LD + k] * A[k * LD + j];
-        Wt[i * LD + j] = acc;
-      }
-      gsync<NT>();
-      for (int t = tid; t < D * (D + 1) / 2; t += NT) {
-        int i, j;
-        tri_index(D, t, i, j);
-        T s = T(0);
-#pragma unroll 4
-        for (int k = 0; k < D; ++k) s += Wt[i * LD + k] * V[j * LD + k];
-        A[i * LD + j] = s;
-        A[j * LD + i] = s;
+    if constexpr (D == 64) {
+      fx64::project<false>(
+          smem_raw + S::V, tid, [&](int i, int j, double& re, double&) { re = A[i * LD + j]; },
+          [&](int i, int j, double re, double) { A[i * LD + j] = re; });
+    } else if constexpr (D == 16) {
+      using namespace fx16;
+      double c[8];
+      Frag q, none;
+      int e = 0, nsw = 0;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) c[u] = A[frag_row(u, tid) * LD + frag_col(u, tid)];
+      const bool finite = fix_matrix<false>(c, c, q, none, e);
+      Result res = kProduct;
+      long long* v = reinterpret_cast<long long*>(vs);
+      if (finite) res = project<false>(q, none, e, v, a.warm != 0, smem_raw + S::V, tid, &dk, &nsw);
+      else if (!a.warm) identity_vectors<false>(v, tid);
+      if (!finite || res != kSame) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          A[frag_row(u, tid) * LD + frag_col(u, tid)] = !finite ? NAN : res == kZero ? 0.0 : word(q[u], e);
       }
     } else {
-      for (int k = tid; k < D; k += NT) {
-        const T w = A[k * LD + k];
-        W[k] = w > T(0) ? w : T(0);
+      if (a.warm) {
+        // A <- V^T C V with the previous eigenvectors
+        for (int e = tid; e < D * D; e += NT) {
+          const int i = e / D, j = e % D;
+          T acc = T(0);
+  #pragma unroll 4
+          for (int k = 0; k < D; ++k) acc += A[i * LD + k] * V[k * LD + j];
+          Wt[i * LD + j] = acc;
+        }
+        gsync<NT>();
+        for (int t = tid; t < D * (D + 1) / 2; t += NT) {
+          int i, j;
+          tri_index(D, t, i, j);
+          T acc = T(0);
+  #pragma unroll 4
+          for (int k = 0; k < D; ++k) acc += V[k * LD + i] * Wt[k * LD + j];
+          A[i * LD + j] = acc;
+          A[j * LD + i] = acc;
+        }
+        gsync<NT>();
+        jacobi_sym<T, D, LD, NT, true, false, true>(A, V, cs, red, tid, &dk);
+      } else {
+        jacobi_sym<T, D, LD, NT, true, true, true>(A, V, cs, red, tid, &dk);
       }
-      gsync<NT>();
-      for (int t = tid; t < D * (D + 1) / 2; t += NT) {
-        int i, j;
-        tri_index(D, t, i, j);
-        T s = T(0);
-#pragma unroll 4
-        for (int k = 0; k < D; ++k) s += W[k] * V[i * LD + k] * V[j * LD + k];
-        A[i * LD + j] = s;
-        A[j * LD + i] = s;
+      for (int e = tid; e < D * D; e += NT) vs[e] = V[(e / D) * LD + (e % D)];
+      if (dk) {
+        // first-order (Daleckii-Krein) reconstruction V M V^T, M = f(Lambda) + L o E
+        dk_matrix_sym<T, D, LD, NT>(A, cs, tid);
+        for (int e = tid; e < D * D; e += NT) {
+          const int i = e / D, j = e % D;
+          T acc = T(0);
+  #pragma unroll 4
+          for (int k = 0; k < D; ++k) acc += V[i * LD + k] * A[k * LD + j];
+          Wt[i * LD + j] = acc;
+        }
+        gsync<NT>();
+        for (int t = tid; t < D * (D + 1) / 2; t += NT) {
+          int i, j;
+          tri_index(D, t, i, j);
+          T s = T(0);
+  #pragma unroll 4
+          for (int k = 0; k < D; ++k) s += Wt[i * LD + k] * V[j * LD + k];
+          A[i * LD + j] = s;
+          A[j * LD + i] = s;
+        }
+      } else {
+        for (int k = tid; k < D; k += NT) {
+          const T w = A[k * LD + k];
+          W[k] = w > T(0) ? w : T(0);
+        }
+        gsync<NT>();
+        for (int t = tid; t < D * (D + 1) / 2; t += NT) {
+          int i, j;
+          tri_index(D, t, i, j);
+          T s = T(0);
+  #pragma unroll 4
+          for (int k = 0; k < D; ++k) s += W[k] * V[i * LD + k] * V[j * LD + k];
+          A[i * LD + j] = s;
+          A[j * LD + i] = s;
+        }
       }
     }
     gsync<NT>();
@@ -499,10 +530,10 @@ cudaError_t launch_pair5(const GenArgs& a, cudaStream_t s) {
   int dev = 0, sms = 0, per = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k5_pair<D>, GroupShape<D>::NT, smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k5_pair<D>, kPairThreads<D>, smem);
   long grid = (long)(sms > 0 ? sms : 1) * (per > 0 ? per : 1);
   if (grid > a.K) grid = a.K;
-  k5_pair<D><<<(unsigned)grid, GroupShape<D>::NT, smem, s>>>(a);
+  k5_pair<D><<<(unsigned)grid, kPairThreads<D>, smem, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -21,31 +21,37 @@
 // All reductions run in a fixed order, so a sweep is bitwise reproducible.
 #include "ve_device.cuh"
 #include "ve_fx16.cuh"
+#include "ve_fx64.cuh"
 #include "ve_internal.h"
 
 namespace ve {
 
 namespace {
 
-template <int D>
+// D = 64 in float64 and double-float (one code for both): the projection in fixed point on the tensor
+// cores (ve_fx64.cuh), by ten warps.
+template <int D, typename T>
+constexpr bool FX64 = D == 64 && std::is_same<T, double>::value;
+
+template <int D, typename T>
 struct PairShape {
   static constexpr int m = ClusterDim<D>::m;
-  static constexpr int NT = GroupShape<D>::NT;
+  static constexpr int NT = FX64<D, T> ? fx64::kThreads : GroupShape<D>::NT;
   static constexpr int LD = GroupShape<D>::LD;
   static constexpr int GPC = GroupShape<D>::GPC;  // groups per CTA
 };
 
 template <int D, typename T>
 struct PairSmem {
-  static constexpr int m = PairShape<D>::m, LD = PairShape<D>::LD;
+  static constexpr int m = PairShape<D, T>::m, LD = PairShape<D, T>::LD;
   static constexpr size_t al(size_t x) { return ((x + 15) / 16) * 16; }
   // per group, in bytes; every array 16-byte aligned
   static constexpr size_t R = 0;                                   // T D*D  (rhs, then rho)
   static constexpr size_t Xs = R + al(sizeof(T) * D * D);          // T D*D  (X_{0,delta})
   static constexpr size_t A = Xs + al(sizeof(T) * D * D);          // T D*LD
-  static constexpr size_t V = A + al(sizeof(T) * D * LD);
-  static constexpr size_t WT = V + al(sizeof(T) * D * LD);         // T D*LD
-  static constexpr size_t CS = WT + al(sizeof(T) * D * LD);        // T D
+  static constexpr size_t V = A + al(sizeof(T) * D * LD);          // T D*LD, or fx64::Smem
+  static constexpr size_t WT = V + (FX64<D, T> ? al(fx64::Smem<false>::bytes) : al(sizeof(T) * D * LD));  // T D*LD
+  static constexpr size_t CS = WT + (FX64<D, T> ? 0 : al(sizeof(T) * D * LD));  // T D
   static constexpr size_t W = CS + al(sizeof(T) * D);              // T D
   static constexpr size_t TR = W + al(sizeof(T) * D);              // T 2*m*m + 2
   static constexpr size_t RED = TR + al(sizeof(T) * (2 * m * m + 2));
@@ -54,10 +60,10 @@ struct PairSmem {
 
 // Arithmetic in T (double, or float in the mixed-precision sweep); the state stays float64.
 template <int D, typename T>
-__global__ void __launch_bounds__(PairShape<D>::NT * PairShape<D>::GPC, GroupShape<D>::MINB)
+__global__ void __launch_bounds__(PairShape<D, T>::NT * PairShape<D, T>::GPC, FX64<D, T> ? 1 : GroupShape<D>::MINB)
     k_pair(const PairArgs a) {
-  constexpr int m = PairShape<D>::m, NT = PairShape<D>::NT, LD = PairShape<D>::LD;
-  constexpr int GPC = PairShape<D>::GPC;
+  constexpr int m = PairShape<D, T>::m, NT = PairShape<D, T>::NT, LD = PairShape<D, T>::LD;
+  constexpr int GPC = PairShape<D, T>::GPC;
   // register-tiled warp products (rgemm16) in float32 only: they compute whole 16 x 16 results
   // where the loops below compute triangles, and float64 / double-float issue is the bound there
   constexpr bool TILE16 = D == 16 && NT == 32 && std::is_same<T, float>::value;
@@ -144,7 +150,7 @@ __global__ void __launch_bounds__(PairShape<D>::NT * PairShape<D>::GPC, GroupSha
     T* vs = reinterpret_cast<T*>(a.vstore) + p * D * D;
     int nsw = 0;
     bool dk = false;  // the eigensolve stopped early: reconstruct with the first-order correction
-    if (a.warm) {
+    if (!FX64<D, T> && a.warm) {
       for (int e = tid; e < D * D; e += NT) V[(e / D) * LD + (e % D)] = vs[e];
       gsync<NT>();
       if (ns_due<T>(a.iter) && TILE16) {
@@ -193,7 +199,11 @@ __global__ void __launch_bounds__(PairShape<D>::NT * PairShape<D>::GPC, GroupSha
       A[j * LD + i] = v;
     }
     gsync<NT>();
-    if (a.warm && TILE16) {
+    if constexpr (FX64<D, T>) {
+      fx64::project<false>(
+          base + S::V, tid, [&](int i, int j, double& re, double&) { re = A[i * LD + j]; },
+          [&](int i, int j, double re, double) { A[i * LD + j] = re; });
+    } else if (a.warm && TILE16) {
       // A <- V^T C V with register-tiled warp products (upper triangle mirrored)
       T acc[2][4];
       rgemm16<T, false, false>(A, LD, V, LD, acc, tid);
@@ -232,63 +242,65 @@ __global__ void __launch_bounds__(PairShape<D>::NT * PairShape<D>::GPC, GroupSha
       atomicAdd(a.stats + 1, 1ull);
       if (dk) atomicAdd(a.stats + 2, 1ull);
     }
-    for (int e = tid; e < D * D; e += NT) vs[e] = V[(e / D) * LD + (e % D)];
-    if (TILE16) {
-      // rho~ = V M V^T (M = f(Lambda) + L o E after a first-order stop, else diag(max(l, 0)))
-      // with register-tiled warp products; the upper triangle is mirrored
-      T acc[2][4];
-      if (dk) {
-        dk_matrix_sym<T, D, LD, NT>(A, cs, tid);
-        rgemm16<T, false, false>(V, LD, A, LD, acc, tid);
-        store16(Wt, LD, acc, tid);
+    if constexpr (!FX64<D, T>) {
+      for (int e = tid; e < D * D; e += NT) vs[e] = V[(e / D) * LD + (e % D)];
+      if (TILE16) {
+        // rho~ = V M V^T (M = f(Lambda) + L o E after a first-order stop, else diag(max(l, 0)))
+        // with register-tiled warp products; the upper triangle is mirrored
+        T acc[2][4];
+        if (dk) {
+          dk_matrix_sym<T, D, LD, NT>(A, cs, tid);
+          rgemm16<T, false, false>(V, LD, A, LD, acc, tid);
+          store16(Wt, LD, acc, tid);
+          __syncwarp();
+          rgemm16<T, false, true>(Wt, LD, V, LD, acc, tid);
+        } else {
+          for (int k = tid; k < D; k += NT) {
+            const T w = A[k * LD + k];
+            W[k] = w > T(0) ? w : T(0);
+          }
+          __syncwarp();
+          rgemm16<T, false, true>(V, LD, V, LD, acc, tid, W);
+        }
         __syncwarp();
-        rgemm16<T, false, true>(Wt, LD, V, LD, acc, tid);
+        store16(A, LD, acc, tid);
+        mirror16<T>(A, nullptr, LD, tid);
+      } else if (dk) {
+        // rho~ = V M V^T with M = f(Lambda) + L o E (dk_stop): Wt = V M, then Wt V^T
+        dk_matrix_sym<T, D, LD, NT>(A, cs, tid);
+        for (int e = tid; e < D * D; e += NT) {
+          const int i = e / D, j = e % D;
+          T acc = T(0);
+  #pragma unroll 4
+          for (int k = 0; k < D; ++k) acc += V[i * LD + k] * A[k * LD + j];
+          Wt[i * LD + j] = acc;
+        }
+        gsync<NT>();
+        for (int t = tid; t < D * (D + 1) / 2; t += NT) {
+          int i, j;
+          tri_index(D, t, i, j);
+          T s = T(0);
+  #pragma unroll 4
+          for (int k = 0; k < D; ++k) s += Wt[i * LD + k] * V[j * LD + k];
+          A[i * LD + j] = s;
+          A[j * LD + i] = s;
+        }
       } else {
         for (int k = tid; k < D; k += NT) {
           const T w = A[k * LD + k];
           W[k] = w > T(0) ? w : T(0);
         }
-        __syncwarp();
-        rgemm16<T, false, true>(V, LD, V, LD, acc, tid, W);
-      }
-      __syncwarp();
-      store16(A, LD, acc, tid);
-      mirror16<T>(A, nullptr, LD, tid);
-    } else if (dk) {
-      // rho~ = V M V^T with M = f(Lambda) + L o E (dk_stop): Wt = V M, then Wt V^T
-      dk_matrix_sym<T, D, LD, NT>(A, cs, tid);
-      for (int e = tid; e < D * D; e += NT) {
-        const int i = e / D, j = e % D;
-        T acc = T(0);
-#pragma unroll 4
-        for (int k = 0; k < D; ++k) acc += V[i * LD + k] * A[k * LD + j];
-        Wt[i * LD + j] = acc;
-      }
-      gsync<NT>();
-      for (int t = tid; t < D * (D + 1) / 2; t += NT) {
-        int i, j;
-        tri_index(D, t, i, j);
-        T s = T(0);
-#pragma unroll 4
-        for (int k = 0; k < D; ++k) s += Wt[i * LD + k] * V[j * LD + k];
-        A[i * LD + j] = s;
-        A[j * LD + i] = s;
-      }
-    } else {
-      for (int k = tid; k < D; k += NT) {
-        const T w = A[k * LD + k];
-        W[k] = w > T(0) ? w : T(0);
-      }
-      gsync<NT>();
-      // rho~ = V diag(max(w, 0)) V^T
-      for (int t = tid; t < D * (D + 1) / 2; t += NT) {
-        int i, j;
-        tri_index(D, t, i, j);
-        T s = T(0);
-#pragma unroll 4
-        for (int k = 0; k < D; ++k) s += W[k] * V[i * LD + k] * V[j * LD + k];
-        A[i * LD + j] = s;
-        A[j * LD + i] = s;
+        gsync<NT>();
+        // rho~ = V diag(max(w, 0)) V^T
+        for (int t = tid; t < D * (D + 1) / 2; t += NT) {
+          int i, j;
+          tri_index(D, t, i, j);
+          T s = T(0);
+  #pragma unroll 4
+          for (int k = 0; k < D; ++k) s += W[k] * V[i * LD + k] * V[j * LD + k];
+          A[i * LD + j] = s;
+          A[j * LD + i] = s;
+        }
       }
     }
     gsync<NT>();
@@ -721,7 +733,7 @@ cudaError_t launch_pair_tc(const PairArgs& a, cudaStream_t s) {
 
 template <int D, typename T>
 cudaError_t launch_pair_t(const PairArgs& a, cudaStream_t s) {
-  constexpr int NT = PairShape<D>::NT, GPC = PairShape<D>::GPC;
+  constexpr int NT = PairShape<D, T>::NT, GPC = PairShape<D, T>::GPC;
   constexpr bool G = GroupShape<D>::GLOBAL;
   const size_t smem = G ? 0 : PairSmem<D, T>::bytes * GPC;
   cudaError_t e = cudaSuccess;
@@ -925,6 +937,9 @@ cudaError_t launch_pair_d(const PairArgs& a, int arith, cudaStream_t s) {
   if constexpr (D == 16) {
     return arith == ARITH_FP32 ? launch_pair_t<D, float>(a, s)
            : arith == ARITH_FP64 || arith == ARITH_DF64 ? launch_pair16(a, s) : cudaErrorInvalidValue;
+  } else if constexpr (D == 64) {
+    return arith == ARITH_FP32 ? launch_pair_t<D, float>(a, s)
+           : arith == ARITH_FP64 || arith == ARITH_DF64 ? launch_pair_t<D, double>(a, s) : cudaErrorInvalidValue;
   } else {
     switch (arith) {
       case ARITH_FP64: return launch_pair_t<D, double>(a, s);
