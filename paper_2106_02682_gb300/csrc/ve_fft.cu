@@ -9,8 +9,8 @@
 // Y_k[e] + i Y_k[e + E] returns both real entry sequences at once.
 //
 // Transform.  Each pass is a length-n DFT (n <= 64) along one axis of the slot array viewed as
-// [A][n][B], done in shared memory by one CTA per (line, chunk of entries): radix-2 in place
-// when n is a power of two, the direct sum otherwise.  A 1-D lattice with N > 64 clusters uses
+// [A][n][B], one CTA per (line, chunk of entries): radix-2 stages in registers when n is a power of
+// two (k_fft_pow2), the direct sum otherwise (k_fft_direct).  A 1-D lattice with N > 64 clusters uses
 // the four-step split N = N1 * N2 with a twiddle between the two passes; the spectrum is then
 // stored digit-reversed (slot c*N2 + e holds k = c + N1*e), which the projection handles through
 // the partner map k -> -k.  A 2-D lattice takes one pass per axis.  Forward sign e^{-i}, no
@@ -57,11 +57,27 @@ struct SpecOf<df64> {
   using R = double;
 };
 
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// a b.  Which of a sum's two products is rounded on its own is written out: left to the compiler it
+// depends on the code around, and a float32 solve's path depends on the last bits of its spectrum
+// (the projections stop at a threshold).
 template <typename V>
 __device__ __forceinline__ V cmul(V a, V b) {
   V r;
-  r.x = a.x * b.x - a.y * b.y;
-  r.y = a.x * b.y + a.y * b.x;
+  r.x = fma_rn(a.x, b.x, -mul_rn(a.y, b.y));
+  r.y = fma_rn(a.y, b.x, mul_rn(a.x, b.y));
+  return r;
+}
+// The same with the other product of the imaginary part rounded (the terms of the direct sum).
+template <typename V>
+__device__ __forceinline__ V cmul_term(V a, V b) {
+  V r;
+  r.x = fma_rn(a.x, b.x, -mul_rn(a.y, b.y));
+  r.y = fma_rn(a.x, b.y, mul_rn(a.y, b.x));
   return r;
 }
 
@@ -73,89 +89,145 @@ __device__ __forceinline__ float tc_hi(float x) { return __uint_as_float(__float
 constexpr int FFT_EC = 32;        // largest number of entries per CTA
 constexpr int FFT_THREADS = 256;
 
-// One pass in precision R (double or float): the spectrum buffers hold C2<R>::type; the real
-// first block row (xin / xout) is always float64.  Twiddles are float64 tables, rounded to R.
+// What the passes share: where element j of a line's column e lies, read and written (with the
+// four-step twiddle on the way out).  The spectrum buffers hold C2<R>::type; the real first block
+// row (xin / xout) is always float64.  Twiddles are float64 tables, rounded to R.
 template <typename R>
-__global__ void __launch_bounds__(FFT_THREADS)
-    k_fft_pass(const double* __restrict__ xin, const typename C2<R>::type* __restrict__ cin,
-               typename C2<R>::type* cout, double* xout, const FftPass ps, const int dir,
-               const int E, const double2* __restrict__ tw, const int EC) {
+struct PassIo {
+  using V = typename C2<R>::type;
+  const double* __restrict__ xin;
+  const V* __restrict__ cin;
+  V* cout;
+  double* xout;
+  const double2* __restrict__ tw;
+  int E;
+  R sg;  // +1 forward, -1 inverse
+
+  __device__ __forceinline__ V load(const FftPass& ps, int la, int lb, int j, int e) const {
+    const long slot = ((long)la * ps.n + j) * ps.B + lb;
+    if (xin) return C2<R>::make((R)xin[slot * 2 * E + e], (R)xin[slot * 2 * E + E + e]);
+    return cin[slot * E + e];
+  }
+  __device__ __forceinline__ V twiddle(double2 wd) const { return C2<R>::make((R)wd.x, sg * (R)wd.y); }
+  __device__ __forceinline__ void store(const FftPass& ps, int la, int lb, int k, int e, V v) const {
+    if (ps.tw_mode) {
+      const int other = (ps.tw_mode == 1) ? lb : la;
+      v = cmul(v, twiddle(tw[ps.tw_off + (int)(((long)k * other) % ps.twN)]));
+    }
+    const long slot = ((long)la * ps.n + k) * ps.B + lb;
+    if (xout) {
+      xout[slot * 2 * E + e] = (double)v.x;
+      xout[slot * 2 * E + E + e] = (double)v.y;
+    } else {
+      cout[slot * E + e] = v;
+    }
+  }
+};
+
+// n = 2^L points: radix-2 decimation in time, three stages at a time in a thread's registers with
+// one exchange through shared memory between them (n <= 64 needs at most two groups of stages).  A
+// thread owns up to eight points of one column; EC columns a CTA, lanes along the entries.  The
+// twiddles 1 and -i of the first three stages cost no multiplication (10 of 12 butterflies).
+// Float64: the float64 pipe bounds it (1216 instructions a column of 64 against 1536 with every
+// product); float32: L2 latency and the float64 <-> float32 conversions of the block row.
+// Measured (4096 clusters, D = 16, a transform of two passes): 61 us in float64, 21 us in float32; 74
+// and 33 us with every stage through shared memory.
+template <typename R, int L>
+__global__ void __launch_bounds__(256) k_fft_pow2(const PassIo<R> io, const FftPass ps, const int EC) {
+  using V = typename C2<R>::type;
+  constexpr int n = 1 << L, RN = n < 8 ? n : 8, L1 = L < 3 ? L : 3, NTH = n / RN;
+  extern __shared__ __align__(16) unsigned char sraw[];
+  V* sbuf = reinterpret_cast<V*>(sraw);
+  const int la = blockIdx.x / ps.B, lb = blockIdx.x % ps.B;
+  const int e = threadIdx.x % EC, g = threadIdx.x / EC;
+  const int ee = blockIdx.y * EC + e;
+  const bool live = ee < io.E;
+  const double2* Wn = io.tw + ps.w_off;  // exp(-2 pi i t / n)
+  V x[RN];
+  // positions RN g + r of the bit-reversed order
+#pragma unroll
+  for (int r = 0; r < RN; ++r)
+    x[r] = live ? io.load(ps, la, lb, bitrev(RN * g + r, L), ee) : C2<R>::make(R(0), R(0));
+#pragma unroll
+  for (int st = 0; st < L1; ++st) {
+    const int half = 1 << st;
+#pragma unroll
+    for (int i0 = 0; i0 < RN; ++i0) {
+      if (i0 & half) continue;
+      const int j = i0 & (half - 1);
+      const V u = x[i0], b = x[i0 + half];
+      V t;
+      if (j == 0) t = b;
+      else if (2 * j == half) t = C2<R>::make(io.sg * b.y, -io.sg * b.x);  // -i b (inverse: i b)
+      else t = cmul(io.twiddle(Wn[j * (n / (2 * half))]), b);
+      x[i0] = C2<R>::make(u.x + t.x, u.y + t.y);
+      x[i0 + half] = C2<R>::make(u.x - t.x, u.y - t.y);
+    }
+  }
+  if constexpr (L <= 3) {
+#pragma unroll
+    for (int r = 0; r < RN; ++r)
+      if (live) io.store(ps, la, lb, r, ee, x[r]);
+  } else {
+    constexpr int G = n / 8;  // points of a group of the later stages: positions q + 8 r
+#pragma unroll
+    for (int r = 0; r < 8; ++r) sbuf[(8 * g + r) * EC + e] = x[r];
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < 8 / G; ++w) {
+      const int q = g + NTH * w;
+      V y[G];
+#pragma unroll
+      for (int r = 0; r < G; ++r) y[r] = sbuf[(q + 8 * r) * EC + e];
+#pragma unroll
+      for (int st = 0; st < L - 3; ++st) {
+        const int half = 1 << st;  // of the group; 8 half points of the line
+#pragma unroll
+        for (int i0 = 0; i0 < G; ++i0) {
+          if (i0 & half) continue;
+          const int j = q + 8 * (i0 & (half - 1));
+          const V u = y[i0], t = cmul(io.twiddle(Wn[j * (n / (16 * half))]), y[i0 + half]);
+          y[i0] = C2<R>::make(u.x + t.x, u.y + t.y);
+          y[i0 + half] = C2<R>::make(u.x - t.x, u.y - t.y);
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < G; ++r)
+        if (live) io.store(ps, la, lb, q + 8 * r, ee, y[r]);
+    }
+  }
+}
+
+// Any n <= 64: the direct sum in shared memory, with the n twiddles there as well (a float64 table
+// entry rounded at every use would cost two conversions at the float64 rate a term).
+template <typename R>
+__global__ void __launch_bounds__(FFT_THREADS) k_fft_direct(const PassIo<R> io, const FftPass ps, const int EC) {
   using V = typename C2<R>::type;
   extern __shared__ __align__(16) unsigned char sraw[];
   V* sbuf = reinterpret_cast<V*>(sraw);
-  const int line = blockIdx.x;
-  const int la = line / ps.B, lb = line % ps.B;
+  const int la = blockIdx.x / ps.B, lb = blockIdx.x % ps.B;
   const int e0 = blockIdx.y * EC;
-  const int ec = min(EC, E - e0);
+  const int ec = min(EC, io.E - e0);
   const int n = ps.n;
-  const bool pow2 = (n & (n - 1)) == 0;
-  const int logn = 31 - __clz(n);
+  V* Wn = sbuf + n * EC;  // exp(-2 pi i t / n)
+  for (int t = threadIdx.x; t < n; t += FFT_THREADS) Wn[t] = io.twiddle(io.tw[ps.w_off + t]);
   for (int idx = threadIdx.x; idx < n * EC; idx += FFT_THREADS) {
     const int j = idx / EC, e = idx % EC;
-    if (e >= ec) continue;
-    const long slot = ((long)la * n + j) * ps.B + lb;
-    V v;
-    if (xin) {
-      v.x = (R)xin[slot * 2 * E + e0 + e];
-      v.y = (R)xin[slot * 2 * E + E + e0 + e];
-    } else {
-      v = cin[slot * E + e0 + e];
-    }
-    const int jj = (pow2 && n > 1) ? bitrev(j, logn) : j;
-    sbuf[jj * EC + e] = v;
+    if (e < ec) sbuf[idx] = io.load(ps, la, lb, j, e0 + e);
   }
   __syncthreads();
-  const double2* Wn = tw + ps.w_off;  // exp(-2 pi i t / n)
-  const V* res = sbuf;
-  const R sg = dir > 0 ? R(-1) : R(1);
-  if (pow2) {
-    for (int half = 1; half < n; half <<= 1) {
-      const int stride = n / (2 * half);
-      for (int idx = threadIdx.x; idx < (n / 2) * EC; idx += FFT_THREADS) {
-        const int e = idx % EC, bf = idx / EC;
-        const int grp = bf / half, j = bf % half;
-        const int i0 = grp * 2 * half + j, i1 = i0 + half;
-        const double2 wd = Wn[j * stride];
-        const V w = C2<R>::make((R)wd.x, sg * (R)wd.y);
-        const V u = sbuf[i0 * EC + e];
-        const V t = cmul(w, sbuf[i1 * EC + e]);
-        sbuf[i0 * EC + e] = C2<R>::make(u.x + t.x, u.y + t.y);
-        sbuf[i1 * EC + e] = C2<R>::make(u.x - t.x, u.y - t.y);
-      }
-      __syncthreads();
-    }
-  } else {
-    V* obuf = sbuf + n * EC;
-    for (int idx = threadIdx.x; idx < n * EC; idx += FFT_THREADS) {
-      const int k = idx / EC, e = idx % EC;
-      V acc = C2<R>::make(R(0), R(0));
-      for (int j = 0; j < n; ++j) {
-        const double2 wd = Wn[(j * k) % n];
-        const V t = cmul(C2<R>::make((R)wd.x, sg * (R)wd.y), sbuf[j * EC + e]);
-        acc.x += t.x;
-        acc.y += t.y;
-      }
-      obuf[idx] = acc;
-    }
-    __syncthreads();
-    res = obuf;
-  }
   for (int idx = threadIdx.x; idx < n * EC; idx += FFT_THREADS) {
     const int k = idx / EC, e = idx % EC;
     if (e >= ec) continue;
-    V v = res[idx];
-    if (ps.tw_mode) {
-      const int other = (ps.tw_mode == 1) ? lb : la;
-      const double2 wd = tw[ps.tw_off + (int)(((long)k * other) % ps.twN)];
-      v = cmul(v, C2<R>::make((R)wd.x, sg * (R)wd.y));
+    V acc = C2<R>::make(R(0), R(0));
+    for (int j = 0, jk = 0; j < n; ++j) {
+      const V t = cmul_term(Wn[jk], sbuf[j * EC + e]);
+      acc.x += t.x;
+      acc.y += t.y;
+      jk += k;
+      if (jk >= n) jk -= n;
     }
-    const long slot = ((long)la * n + k) * ps.B + lb;
-    if (xout) {
-      xout[slot * 2 * E + e0 + e] = (double)v.x;
-      xout[slot * 2 * E + E + e0 + e] = (double)v.y;
-    } else {
-      cout[slot * E + e0 + e] = v;
-    }
+    io.store(ps, la, lb, k, e0 + e, acc);
   }
 }
 
@@ -718,14 +790,20 @@ cudaError_t run_pass_t(const FftPlan& p, const FftPass& ps, int dir, const doubl
     ec = FFT_EC;
     while (ec > 8 && lines * ((p.E + ec - 1) / ec) < 304) ec /= 2;
   }
-  const size_t smem = sizeof(V) * ps.n * ec * (pow2 ? 1 : 2);
-  static unsigned long long mask = 0;
-  cudaError_t e = smem_once(k_fft_pass<R>, 2 * sizeof(V) * 64 * FFT_EC, mask);
-  if (e != cudaSuccess) return e;
-  dim3 grid((unsigned)lines, (unsigned)((p.E + ec - 1) / ec));
-  k_fft_pass<R><<<grid, FFT_THREADS, smem, s>>>(xin, reinterpret_cast<const V*>(cin),
-                                                reinterpret_cast<V*>(cout), xout, ps, dir, p.E, tw,
-                                                ec);
+  const PassIo<R> io = {xin, reinterpret_cast<const V*>(cin), reinterpret_cast<V*>(cout), xout, tw, p.E,
+                        dir > 0 ? R(-1) : R(1)};
+  const dim3 grid((unsigned)lines, (unsigned)((p.E + ec - 1) / ec));
+  const size_t smem = sizeof(V) * ps.n * ec;  // at most 32 KB (33 with the direct sum's twiddles)
+  const int threads = ps.n > 8 ? ec * (ps.n / 8) : ec;
+  switch (pow2 ? ps.n : 0) {
+    case 2: k_fft_pow2<R, 1><<<grid, threads, 0, s>>>(io, ps, ec); break;
+    case 4: k_fft_pow2<R, 2><<<grid, threads, 0, s>>>(io, ps, ec); break;
+    case 8: k_fft_pow2<R, 3><<<grid, threads, 0, s>>>(io, ps, ec); break;
+    case 16: k_fft_pow2<R, 4><<<grid, threads, smem, s>>>(io, ps, ec); break;
+    case 32: k_fft_pow2<R, 5><<<grid, threads, smem, s>>>(io, ps, ec); break;
+    case 64: k_fft_pow2<R, 6><<<grid, threads, smem, s>>>(io, ps, ec); break;
+    default: k_fft_direct<R><<<grid, FFT_THREADS, smem + sizeof(V) * ps.n, s>>>(io, ps, ec);
+  }
   return cudaGetLastError();
 }
 
