@@ -179,7 +179,7 @@ int ve_get_status(ve_handle* h, ve_status* out);
 
 /* Per-stage timing.  ve_profile(h, 1) clears the accumulators and makes every following sweep
  * run uncaptured with CUDA events (on the handle's stream) around each of its VE_NSTAGE stages:
- * 0 pair pass, 1 rho_0 update, 2 Lambda1/Lambda2 update, 3 status, 4 forward block DFT,
+ * 0 pair pass, 1 rho_0 update, 2 Lambda1/Lambda2 update and status (one launch; 3 is empty), 4 forward block DFT,
  * 5 per-wavevector projection, 6 inverse block DFT.  ve_profile(h, 0) returns to graph replay.
  * ve_profile_read writes accumulated milliseconds and kernel launches per stage (arrays of
  * VE_NSTAGE, host).  Errors: VE_EINVAL, VE_ECUDA. */

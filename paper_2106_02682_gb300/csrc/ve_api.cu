@@ -161,6 +161,9 @@ struct ve_handle {
   ve_options opt;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
+  // the multiplier update and the status run beside the X step (issue_sweep)
+  cudaStream_t side = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
   int device = 0;
   FftPlan plan;
   int P = 0;
@@ -170,7 +173,7 @@ struct ve_handle {
   double *state = nullptr, *rho0 = nullptr, *rt = nullptr, *lam = nullptr, *lam1 = nullptr,
          *lam2 = nullptr, *X = nullptr;
   double* rho0_partial = nullptr;
-  double *a1r = nullptr, *a2r = nullptr, *part = nullptr, *part2 = nullptr, *hb = nullptr,
+  double *a1r = nullptr, *a2r = nullptr, *part = nullptr, *hb = nullptr,
          *H0 = nullptr, *lmin_pairs = nullptr, *lmin_k = nullptr, *lmin0 = nullptr;
   int *hslot = nullptr, *neg = nullptr, *canon = nullptr;
   int ncanon = 0;
@@ -262,7 +265,6 @@ SmallArgs small_args(ve_handle* h) {
   a.a1r = h->a1r;
   a.a2r = h->a2r;
   a.part = h->part;
-  a.part2 = h->part2;
   a.st = h->dst;
   a.rho0_partial = h->rho0_partial;
   a.ptie = h->ptie;
@@ -296,10 +298,20 @@ cudaError_t issue_sweep(ve_handle* h, int arith, bool warm) {
   if ((e = mark(1)) != cudaSuccess) return e;
   if ((e = launch_rho0(sa, s)) != cudaSuccess) return e;
   if ((e = mark(2)) != cudaSuccess) return e;
-  if ((e = launch_dual12(sa, s)) != cudaSuccess) return e;
+  // Lambda1, Lambda2 and the status need rho_0 only, and nothing before the next sweep needs them.
+  // Small instances leave SMs idle and run them on a branch beside the X step; large ones in line,
+  // where the branch costs more than its 10 us (measured, us a sweep, branch / line: 16 clusters 60
+  // / 66, 50 clusters 153 / 159, 2048 clusters 253 / 230, 4096 clusters 372 / 345).
+  const bool beside = !h->prof && h->Pc <= 2 * big_grid();
+  const cudaStream_t q = beside ? h->side : s;
+  if (beside) {
+    if ((e = cudaEventRecord(h->fork, s)) != cudaSuccess) return e;
+    if ((e = cudaStreamWaitEvent(q, h->fork, 0)) != cudaSuccess) return e;
+  }
+  if ((e = launch_dual_status(sa, q)) != cudaSuccess) return e;
   if ((e = mark(3)) != cudaSuccess) return e;
-  if ((e = launch_status(sa, s)) != cudaSuccess) return e;
   if ((e = mark(4)) != cudaSuccess) return e;
+  if (beside && (e = cudaEventRecord(h->join, q)) != cudaSuccess) return e;
   double2* spec = nullptr;
   if ((e = fft_forward(h->plan, h->X, h->specA, h->specB, h->tw, &spec, fp32, s)) != cudaSuccess)
     return e;
@@ -309,12 +321,13 @@ cudaError_t issue_sweep(ve_handle* h, int arith, bool warm) {
                              h->prof ? h->jstats + 3 : nullptr)) != cudaSuccess)
       return e;
   } else if ((e = launch_xproj(h->plan, spec, h->canon, arith, h->vk[v], warm ? 1 : 0, s,
-                              h->prof ? h->jstats + 3 : nullptr, h->gws, &h->dst->iter)) != cudaSuccess) {
+                              h->prof ? h->jstats + 3 : nullptr, h->gws, &h->dst->sweep)) != cudaSuccess) {
     return e;
   }
   if ((e = mark(6)) != cudaSuccess) return e;
   if ((e = fft_inverse(h->plan, spec, h->specA, h->specB, h->X, h->tw, fp32, s)) != cudaSuccess)
     return e;
+  if (beside && (e = cudaStreamWaitEvent(s, h->join, 0)) != cudaSuccess) return e;
   return mark(7);
 }
 
@@ -518,7 +531,6 @@ int ve_create(const ve_lattice* lattice, const ve_cluster* cluster, const ve_ham
   const size_t o_a1r = take(sizeof(double) * P * mm);
   const size_t o_a2r = take(sizeof(double) * P * mm);
   const size_t o_part = take(sizeof(double) * 2 * P);
-  const size_t o_part2 = take(sizeof(double) * P);
   const size_t o_r0p = take(sizeof(double) * 128 * mm);
   const size_t o_hb = take(sizeof(double) * (nb > 0 ? nb : 1) * DD);
   const size_t o_H0 = take(sizeof(double) * mm);
@@ -568,7 +580,6 @@ int ve_create(const ve_lattice* lattice, const ve_cluster* cluster, const ve_ham
   h->a1r = (double*)(base + o_a1r);
   h->a2r = (double*)(base + o_a2r);
   h->part = (double*)(base + o_part);
-  h->part2 = (double*)(base + o_part2);
   h->rho0_partial = (double*)(base + o_r0p);
   h->hb = (double*)(base + o_hb);
   h->H0 = (double*)(base + o_H0);
@@ -623,6 +634,12 @@ int ve_create(const ve_lattice* lattice, const ve_cluster* cluster, const ve_ham
     }
     h->own_stream = true;
   }
+  if (cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&h->fork, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&h->join, cudaEventDisableTiming) != cudaSuccess) {
+    ve_destroy(h);
+    return VE_ECUDA;
+  }
   // host staging: initial state (Sec. 4), Hamiltonian blocks, index tables
   std::vector<double> st(h->state_bytes / sizeof(double), 0.0);
   for (int i = 0; i < m; ++i) st[(size_t)i * m + i] = 1.0 / m;
@@ -676,7 +693,7 @@ int ve_create(const ve_lattice* lattice, const ve_cluster* cluster, const ve_ham
     return VE_ECUDA;
   }
   *h->hst = ds;
-  const int launches[VE_NSTAGE] = {1, 1, 1, 1, h->plan.npass, 1, h->plan.npass};
+  const int launches[VE_NSTAGE] = {1, 1, 1, 0, h->plan.npass, 1, h->plan.npass};
   for (int i = 0; i < VE_NSTAGE; ++i) h->stage_launches[i] = launches[i];
   *out = h;
   return VE_OK;
@@ -693,6 +710,9 @@ void ve_destroy(ve_handle* h) {
   for (int i = 0; i <= VE_NSTAGE; ++i)
     if (h->ev[i]) cudaEventDestroy(h->ev[i]);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
+  if (h->side) cudaStreamDestroy(h->side);
+  if (h->fork) cudaEventDestroy(h->fork);
+  if (h->join) cudaEventDestroy(h->join);
   if (h->hst) cudaFreeHost(h->hst);
   if (h->dev) cudaFree(h->dev);
   if (h->tcmem) cudaFree(h->tcmem);

@@ -80,6 +80,8 @@ struct DevStatus {
   double h0rho0;  // Tr[H_0 rho_0] of the current sweep
   unsigned int done;  // CTAs of the running multi-CTA reduction finished (0 between kernels)
   unsigned int pad;
+  long long sweep;    // iter after the running sweep, set by the rho_0 update (iter itself moves on
+                      // a branch of its own beside the X step)
 };
 
 struct SmallArgs {
@@ -93,7 +95,6 @@ struct SmallArgs {
   const double* a1r;
   const double* a2r;
   const double* part;
-  double* part2;  // P: ||A1 rho - rho0||^2 + ||A2 rho - rho0||^2
   // P: for the canonical member of {delta, -delta} the pair index of the other, -1 when
   // -delta = delta, -2 for the member whose Lambda1, Lambda2 its partner writes; or nullptr
   const int* ptie;
@@ -114,8 +115,7 @@ size_t bound_ws_bytes(int D);
 cudaError_t launch_pair(const PairArgs& a, int arith, cudaStream_t s);
 // rho_0 update: two launches (chunk sums over delta, then one CTA), fixed reduction order.
 cudaError_t launch_rho0(const SmallArgs& a, cudaStream_t s);
-cudaError_t launch_dual12(const SmallArgs& a, cudaStream_t s);
-cudaError_t launch_status(const SmallArgs& a, cudaStream_t s);
+cudaError_t launch_dual_status(const SmallArgs& a, cudaStream_t s);
 
 // ------------------------------------------------------------------ block DFT over delta
 // The first block row is viewed as a row-major array [A][n][B] of slots (delta, or wavevector

@@ -15,9 +15,8 @@
 // k_rho0     : rho_0 update (Eq. (rhoiUpdate), translation-invariant form) with the trace
 //              shift, and X'_00 = X_00 - eps G_00[rho_0]: every CTA sums a chunk of offsets, the
 //              last CTA to finish adds the chunk sums and updates rho_0.
-// k_dual12   : Lambda1/Lambda2 updates (they need the new rho_0) and their feasibility terms.
-// k_status   : energy per spin, Eq. (feasErr), |energy change|, residual (CTA sums, then
-//              the last CTA).
+// k_dual_status : Lambda1/Lambda2 updates (they need the new rho_0); energy per spin, Eq. (feasErr),
+//              |energy change|, residual (CTA sums, then the last CTA).
 // All reductions run in a fixed order, so a sweep is bitwise reproducible.
 #include "ve_device.cuh"
 #include "ve_fx16.cuh"
@@ -754,57 +753,62 @@ cudaError_t launch_pair_t(const PairArgs& a, cudaStream_t s) {
 // RHO0_CHUNKS CTAs each sum a contiguous range of offsets delta of nu A1[rho_{0,delta}] +
 // Lambda1_{0,delta} (m*m entries); the last CTA to finish (a counter in the status block) adds
 // the chunk sums in order.  Both orders are fixed, so the result is reproducible bit for bit.
+// Latency bounds it (a float64 add of a lone warp takes 64 cycles), and the X step waits for it: up
+// to RHO0_CHUNKS offsets one CTA forms the chunks' terms itself, added in the same order, without
+// the counter's round trip; what does not depend on the sums is read before them.
 constexpr int RHO0_CHUNKS = 128;
 
 __global__ void __launch_bounds__(256) k_rho0(const SmallArgs a, double* partial) {
-  const int mm = a.m * a.m;
-  const long per = (a.P + RHO0_CHUNKS - 1) / RHO0_CHUNKS;
-  const long lo = blockIdx.x * per, hi = min((long)a.P, lo + per);
+  const int m = a.m, mm = m * m, D = a.D;
   // threads: (entry, sub-range) with 256 / mm sub-ranges per chunk
   const int subs = 256 / mm;
   __shared__ double S[256];
   const int t = threadIdx.x;
-  double acc = 0.0;
-  if (t < subs * mm) {
-    const int idx = t % mm, c = t / mm;
-    for (long p = lo + c; p < hi; p += subs) acc += a.nu * a.a1r[p * mm + idx] + a.lam1[p * mm + idx];
-  }
-  S[t] = acc;
-  __syncthreads();
+  const int idx = t % mm, c = t / mm;
+  auto term = [&](long p) { return a.nu * a.a1r[p * mm + idx] + a.lam1[p * mm + idx]; };
+  // H'_0 = H_0 - sum_a X_{(a,b),(a,d)}  (Eq. (effHam) with matrix units)
+  double h0 = 0.0, h0p = 0.0;
   if (t < mm) {
-    double s = 0.0;
-    for (int c = 0; c < subs; ++c) s += S[c * mm + t];
-    partial[blockIdx.x * mm + t] = s;
-  }
-  __threadfence();
-  __shared__ bool last;
-  __syncthreads();
-  if (t == 0) last = atomicAdd(&a.st->done, 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  // the last CTA: rho_0 from the chunk sums (read past L1: other CTAs wrote them), each entry
-  // summed by subs threads over interleaved chunks, then in order over the threads
-  {
-    double acc2 = 0.0;
-    if (t < subs * mm) {
-      const int idx = t % mm, c0 = t / mm;
-      for (int c = c0; c < RHO0_CHUNKS; c += subs) acc2 += __ldcg(partial + c * mm + idx);
-    }
-    S[t] = acc2;
-  }
-  __syncthreads();
-  __shared__ double rp[256];
-  __shared__ double red[8];
-  const int m = a.m, D = a.D;
-  if (t < mm) {
-    double s = 0.0;
-    for (int c = 0; c < subs; ++c) s += S[c * mm + t];
-    // H'_0 = H_0 - sum_a X_{(a,b),(a,d)}  (Eq. (effHam) with matrix units)
     const int b = t / m, d = t % m;
     double hx = 0.0;
     for (int x = 0; x < m; ++x) hx += a.X[(x * m + b) * D + (x * m + d)];
-    const double h0p = a.H0[t] - hx;
+    h0 = a.H0[t];
+    h0p = h0 - hx;
+  }
+  double acc = 0.0;
+  if (gridDim.x == 1) {
+    for (long p = c; p < a.P; p += subs) acc += term(p);
+  } else {
+    const long per = (a.P + RHO0_CHUNKS - 1) / RHO0_CHUNKS;
+    const long lo = blockIdx.x * per, hi = min((long)a.P, lo + per);
+    for (long p = lo + c; p < hi; p += subs) acc += term(p);
+    S[t] = acc;
+    __syncthreads();
+    if (t < mm) {
+      double s = 0.0;
+      for (int k = 0; k < subs; ++k) s += S[k * mm + t];
+      partial[blockIdx.x * mm + t] = s;
+    }
+    __threadfence();
+    __shared__ bool last;
+    __syncthreads();
+    if (t == 0) last = atomicAdd(&a.st->done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    // the last CTA: rho_0 from the chunk sums (read past L1: other CTAs wrote them), each entry
+    // summed by subs threads over interleaved chunks, then in order over the threads
+    acc = 0.0;
+    for (int k = c; k < RHO0_CHUNKS; k += subs) acc += __ldcg(partial + k * mm + idx);
+  }
+  S[t] = acc;
+  __syncthreads();
+  __shared__ double rp[256];
+  __shared__ double red[8];
+  if (t < mm) {
+    const int live = gridDim.x == 1 && a.P < subs ? a.P : subs;  // the others hold zeros
+    double s = 0.0;
+    for (int k = 0; k < live; ++k) s += S[k * mm + t];
     rp[t] = (s - h0p) / (a.nu * (a.N - 1));
   }
   __syncthreads();
@@ -813,98 +817,100 @@ __global__ void __launch_bounds__(256) k_rho0(const SmallArgs a, double* partial
   const double z = (1.0 - tr) / m;
   __syncthreads();
   if (t < mm) {
-    const int b = t / m, d = t % m;
-    rp[t] = rp[t] + (b == d ? z : 0.0);
+    const double r = rp[t] + (t / m == t % m ? z : 0.0);
+    rp[t] = r;
+    a.rho0[t] = r;
   }
   __syncthreads();
-  if (t < mm) a.rho0[t] = rp[t];
   // X'_00 = X_00 - eps G_00[rho_0], G_00 entry (a,b),(c,d) = delta_ac rho0_{d,b}
-  for (int e = t; e < D * D; e += 256) {
-    const int i = e / D, j = e % D;
-    const int pa = i / m, pb = i % m, pc = j / m, pd = j % m;
-    if (pa == pc) a.X[e] -= a.eps * rp[pd * m + pb];
+  for (int u = t; u < m * mm; u += 256) {
+    const int pa = u / mm, pb = (u / m) % m, pd = u % m;
+    a.X[(pa * m + pb) * D + (pa * m + pd)] -= a.eps * rp[pd * m + pb];
   }
   // Tr[H_0 rho_0]
   double h = 0.0;
-  if (t < mm) h = a.H0[t] * rp[(t % m) * m + (t / m)];
+  if (t < mm) h = h0 * rp[(t % m) * m + (t / m)];
   h = gsum<256>(h, red);
   if (t == 0) {
     a.st->h0rho0 = h;
     a.st->done = 0u;  // ready for the next sweep
+    a.st->sweep = a.st->iter + 1;
   }
 }
 
-// ---------------------------------------------------------------- Lambda1, Lambda2
+// ---------------------------------------------------------------- Lambda1, Lambda2, status
 // One warp per pair offset.  With ties (see k_pair) the canonical member of {delta, -delta}
 // also writes the other's multipliers, Lambda1_{-delta} = Lambda2_delta and Lambda2_{-delta} =
-// Lambda1_delta, so the two stay exact swap images.
-__global__ void k_dual12(const SmallArgs a) {
-  const int lane = threadIdx.x & 31;
-  const long w = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+// Lambda1_delta, so the two stay exact swap images (and the offset counts twice in the sums).  Every
+// CTA adds up its offsets' residual and energy terms; the last one to finish adds the CTA sums in
+// order and writes the status block: one launch for what were two (8 + 13 us, latency).
+constexpr int DUAL_CTAS = 128, DUAL_THREADS = 256;
+
+__global__ void __launch_bounds__(DUAL_THREADS) k_dual_status(const SmallArgs a, double* partial) {
+  __shared__ double red[DUAL_THREADS / 32][3];
+  const int lane = threadIdx.x & 31, wc = threadIdx.x >> 5;
   const int mm = a.m * a.m;
-  if (w >= a.P) return;
-  const long tie = a.ptie ? a.ptie[w] : -1;
-  if (tie == -2) return;  // uniform over the warp
-  double s = 0.0;
-  for (int idx = lane; idx < mm; idx += 32) {
-    const double r0 = a.rho0[idx];
-    const double d1 = a.a1r[w * mm + idx] - r0;
-    const double d2 = a.a2r[w * mm + idx] - r0;
-    const double n1 = a.lam1[w * mm + idx] + a.nu * d1;
-    const double n2 = a.lam2[w * mm + idx] + a.nu * d2;
-    a.lam1[w * mm + idx] = n1;
-    a.lam2[w * mm + idx] = n2;
-    if (tie >= 0) {
-      a.lam1[tie * mm + idx] = n2;
-      a.lam2[tie * mm + idx] = n1;
+  const long warps = (long)gridDim.x * (DUAL_THREADS / 32);
+  double rr = 0.0, en = 0.0, ff = 0.0;
+  for (long w = (long)blockIdx.x * (DUAL_THREADS / 32) + wc; w < a.P; w += warps) {
+    const long tie = a.ptie ? a.ptie[w] : -1;
+    if (tie == -2) continue;  // uniform over the warp
+    double s = 0.0;
+    for (int idx = lane; idx < mm; idx += 32) {
+      const double r0 = a.rho0[idx];
+      const double d1 = a.a1r[w * mm + idx] - r0;
+      const double d2 = a.a2r[w * mm + idx] - r0;
+      const double n1 = a.lam1[w * mm + idx] + a.nu * d1;
+      const double n2 = a.lam2[w * mm + idx] + a.nu * d2;
+      a.lam1[w * mm + idx] = n1;
+      a.lam2[w * mm + idx] = n2;
+      if (tie >= 0) {
+        a.lam1[tie * mm + idx] = n2;
+        a.lam2[tie * mm + idx] = n1;
+      }
+      s += d1 * d1 + d2 * d2;
     }
-    s += d1 * d1 + d2 * d2;
+    const double c = tie >= 0 ? 2.0 : 1.0;
+    ff = fma(c, s, ff);
+    if (lane == 0) {
+      rr = fma(c, a.part[w * 2 + 0], rr);
+      en = fma(c, a.part[w * 2 + 1], en);
+    }
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  for (int o = 16; o > 0; o >>= 1) ff += __shfl_xor_sync(0xffffffffu, ff, o);
   if (lane == 0) {
-    a.part2[w] = s;
-    if (tie >= 0) a.part2[tie] = s;
+    red[wc][0] = rr;
+    red[wc][1] = en;
+    red[wc][2] = ff;
   }
-}
-
-// ---------------------------------------------------------------- status
-// STATUS_CTAS CTAs each sum a contiguous range of offsets (float64 adds are spread over as many
-// SMs); the last CTA to finish adds the CTA sums in order and writes the status block.
-constexpr int STATUS_CTAS = 32;
-
-__global__ void __launch_bounds__(256) k_status(const SmallArgs a, double* partial) {
-  __shared__ double red[8];
-  const long per = (a.P + STATUS_CTAS - 1) / STATUS_CTAS;
-  const long lo = blockIdx.x * per, hi = min((long)a.P, lo + per);
-  double rr = 0.0, en = 0.0, ff = 0.0;
-  for (long p = lo + threadIdx.x; p < hi; p += 256) {
-    rr += a.part[p * 2 + 0];
-    en += a.part[p * 2 + 1];
-    ff += a.part2[p];
-  }
-  rr = gsum<256>(rr, red);
-  en = gsum<256>(en, red);
-  ff = gsum<256>(ff, red);
-  if (threadIdx.x == 0) {
-    partial[blockIdx.x * 3 + 0] = rr;
-    partial[blockIdx.x * 3 + 1] = en;
-    partial[blockIdx.x * 3 + 2] = ff;
+  __syncthreads();
+  const int t = threadIdx.x;
+  if (t < 3) {
+    double v = 0.0;
+    for (int k = 0; k < DUAL_THREADS / 32; ++k) v += red[k][t];
+    partial[blockIdx.x * 3 + t] = v;
   }
   __threadfence();
   __shared__ bool last;
   __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(&a.st->done, 1u) == gridDim.x - 1;
+  if (t == 0) last = atomicAdd(&a.st->done, 1u) == gridDim.x - 1;
   __syncthreads();
   if (!last) return;
   __threadfence();
-  const int t = threadIdx.x;
-  rr = t < STATUS_CTAS ? __ldcg(partial + t * 3 + 0) : 0.0;
-  en = t < STATUS_CTAS ? __ldcg(partial + t * 3 + 1) : 0.0;
-  ff = t < STATUS_CTAS ? __ldcg(partial + t * 3 + 2) : 0.0;
-  rr = gsum<256>(rr, red);
-  en = gsum<256>(en, red);
-  ff = gsum<256>(ff, red);
+  if (t >= 32) return;
+  rr = en = ff = 0.0;
+  for (int k = t; k < (int)gridDim.x; k += 32) {
+    rr += __ldcg(partial + k * 3 + 0);
+    en += __ldcg(partial + k * 3 + 1);
+    ff += __ldcg(partial + k * 3 + 2);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    rr += __shfl_xor_sync(0xffffffffu, rr, o);
+    en += __shfl_xor_sync(0xffffffffu, en, o);
+    ff += __shfl_xor_sync(0xffffffffu, ff, o);
+  }
   if (t == 0) {
     DevStatus* st = a.st;
     st->done = 0u;
@@ -976,19 +982,13 @@ int big_grid() {
 }
 
 cudaError_t launch_rho0(const SmallArgs& a, cudaStream_t s) {
-  k_rho0<<<RHO0_CHUNKS, 256, 0, s>>>(a, a.rho0_partial);
+  k_rho0<<<a.P <= RHO0_CHUNKS ? 1 : RHO0_CHUNKS, 256, 0, s>>>(a, a.rho0_partial);
   return cudaGetLastError();
 }
 
-cudaError_t launch_dual12(const SmallArgs& a, cudaStream_t s) {
-  const long threads = (long)a.P * 32;
-  const unsigned blocks = (unsigned)((threads + 255) / 256);
-  k_dual12<<<blocks, 256, 0, s>>>(a);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_status(const SmallArgs& a, cudaStream_t s) {
-  k_status<<<STATUS_CTAS, 256, 0, s>>>(a, a.rho0_partial);
+cudaError_t launch_dual_status(const SmallArgs& a, cudaStream_t s) {
+  const long need = ((long)a.P + DUAL_THREADS / 32 - 1) / (DUAL_THREADS / 32);
+  k_dual_status<<<(unsigned)(need < DUAL_CTAS ? need : DUAL_CTAS), DUAL_THREADS, 0, s>>>(a, a.rho0_partial);
   return cudaGetLastError();
 }
 
