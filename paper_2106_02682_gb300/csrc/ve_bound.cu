@@ -14,6 +14,7 @@
 // remaining off-diagonal part, a lower bound by Weyl's inequality whether or not the Jacobi
 // sweeps converged; minima pass a NaN on (nan_min), so a non-finite state cannot certify.
 #include "ve_device.cuh"
+#include "ve_fx16.cuh"
 #include "ve_internal.h"
 
 namespace ve {
@@ -76,6 +77,47 @@ __global__ void __launch_bounds__(BShape<D>::NT * BShape<D>::GPC, GroupShape<D>:
     // Weyl: the rotated matrix is diag + E, so lmin >= min diag - ||E||_2 >= min diag - ||E||_F
     if (tid == 0) a.lmin_pairs[p] = w - sqrt(off);
     gsync<NT>();
+  }
+}
+
+// lmin(K_delta) for D = 16: one warp a pair, in fixed point (ve_fx16.cuh).
+__global__ void __launch_bounds__(32, 16) k_bound_pairs16(const BoundArgs a) {
+  using namespace fx16;
+  constexpr int D = 16, m = 4, mm = 16;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr size_t fx = D * D * sizeof(double);
+  double* Xs = reinterpret_cast<double*>(smem_raw);
+  const int lane = threadIdx.x;
+  for (long p = blockIdx.x; p < a.P; p += gridDim.x) {
+    const long dl = p + 1;
+    const double* Xb = a.X + dl * D * D;
+    const int hs = a.hslot[dl];
+    const double* Hb = hs >= 0 ? a.hb + (long)hs * D * D : nullptr;
+    const double* l1 = a.lam1 + p * mm;
+    const double* l1n = a.lam1 + (long)(a.neg[dl] - 1) * mm;
+    for (int e = lane; e < D * D; e += 32) Xs[e] = Xb[e];
+    __syncwarp();
+    double c[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int i = frag_row(k, lane), j = frag_col(k, lane);
+      const int pa = i / m, pb = i % m, pc = j / m, pd = j % m;
+      c[k] = Hb ? Hb[i * D + j] : 0.0;
+      c[k] -= Xs[(pa * m + pc) * D + (pd * m + pb)] + Xs[(pc * m + pa) * D + (pb * m + pd)];
+      if (pb == pd) c[k] += l1[pa * m + pc];
+      if (pa == pc) c[k] += l1n[pb * m + pd];
+    }
+    Frag q, none;
+    int e = 0;
+    double w = NAN;
+    if (fix_matrix<false>(c, c, q, none, e)) {
+      add_adjoint<false>(q, none, smem_raw + fx, lane);
+      e -= 1;
+      normalise<false>(q, none, e);
+      w = lowest<false>(q, none, e, smem_raw + fx, lane);
+    }
+    if (lane == 0) a.lmin_pairs[p] = w;
+    __syncwarp();
   }
 }
 
@@ -266,6 +308,18 @@ __global__ void __launch_bounds__(PShape<n, T>::NT * PShape<n, T>::GPC)
 }
 
 
+cudaError_t launch_bound16(const BoundArgs& a, cudaStream_t s) {
+  const size_t smem = 256 * sizeof(double) + fx16::Smem<false>::bytes + fx16::Smem<false>::vectors;
+  static unsigned long long mask = 0;
+  cudaError_t e = smem_once(k_bound_pairs16, smem, mask);
+  if (e != cudaSuccess) return e;
+  const long res = resident_grid((const void*)k_bound_pairs16, 32, smem);
+  k_bound_pairs16<<<(unsigned)(a.P < res ? a.P : res), 32, smem, s>>>(a);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  k_bound_k0<4><<<1, 256, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
 template <int D>
 cudaError_t launch_bound_t(const BoundArgs& a, cudaStream_t s) {
   constexpr int NT = BShape<D>::NT, GPC = BShape<D>::GPC, m = BShape<D>::m;
@@ -333,7 +387,7 @@ cudaError_t launch_proj_herm_t(const double* in, double* out, long count, unsign
 cudaError_t launch_bound(const BoundArgs& a, cudaStream_t s) {
   switch (a.D) {
     case 4: return launch_bound_t<4>(a, s);
-    case 16: return launch_bound_t<16>(a, s);
+    case 16: return launch_bound16(a, s);
     case 64: return launch_bound_t<64>(a, s);
     case 256: return launch_bound_t<256>(a, s);
     default: return cudaErrorInvalidValue;

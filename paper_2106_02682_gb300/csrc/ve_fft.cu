@@ -548,10 +548,31 @@ __global__ void __launch_bounds__(GroupShape<D>::NT * GroupShape<D>::GPC, GroupS
   }
 }
 
+// Block 4 C_k (unnormalised, exactly Hermitian) of slots s, s2 = -k of a D = 16 spectrum as fixed
+// point.  A lane's rows g and g + 8 of its columns are exactly the entry pairs e, e + E that share
+// a packed complex sequence.  false when an entry is not finite.
+__device__ __forceinline__ bool unpack16(const double2* z1, const double2* z2, fx16::Frag& ar, fx16::Frag& ai, int& ea,
+                                         unsigned char* sm, int lane) {
+  double cr[8], ci[8];  // 2 C_k
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int k = (u & 1) + 4 * (u >> 1);  // fragment element of row g; k + 2 is row g + 8
+    const int e = fx16::frag_row(k, lane) * 16 + fx16::frag_col(k, lane);
+    const double2 z = z1[e], zz = z2[e];  // conj(zz) taken below
+    cr[k] = z.x + zz.x;                   // z + conj(zz)
+    ci[k] = z.y - zz.y;
+    cr[k + 2] = z.y + zz.y;               // (z - conj(zz)) / i
+    ci[k + 2] = zz.x - z.x;
+  }
+  if (!fx16::fix_matrix<true>(cr, ci, ar, ai, ea)) return false;
+  fx16::add_adjoint<true>(ar, ai, sm, lane);
+  fx16::normalise<true>(ar, ai, ea);
+  return true;
+}
+
 // The same projection for D = 16 in float64 and double-float (one code for both: it is the faster
 // of the two and accurate to float64): one warp per canonical wavevector, in the fixed-point form of
-// ve_fx16.cuh.  A lane's rows g and g + 8 of its columns are exactly the entry pairs e, e + E
-// that share a packed complex sequence, so the block is unpacked and packed back in registers.
+// ve_fx16.cuh.  The block is unpacked (unpack16) and packed back in registers.
 // Without a store the eigenvectors stay in shared memory.
 // Measured (4096 clusters, 2049 blocks): 149 us; 1000 us as float64 Jacobi sweeps (float64 pipe 85 %
 // busy).  Bound by issue: 26k integer, MMA and float32 instructions a block at 42 % of the issue slots
@@ -573,28 +594,12 @@ __global__ void __launch_bounds__(32, 16)
         vstore ? vstore + (long)s * 512 : reinterpret_cast<long long*>(smem_raw + fx16::Smem<true>::bytes);
     Frag ar, ai;
     int ea;
-    bool finite;
-    {
-      double cr[8], ci[8];  // 2 C_k
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int k = (u & 1) + 4 * (u >> 1);  // fragment element of row g; k + 2 is row g + 8
-        const int e = fx16::frag_row(k, lane) * 16 + fx16::frag_col(k, lane);
-        const double2 z = z1[e], zz = z2[e];  // conj(zz) taken below
-        cr[k] = z.x + zz.x;                   // z + conj(zz)
-        ci[k] = z.y - zz.y;
-        cr[k + 2] = z.y + zz.y;               // (z - conj(zz)) / i
-        ci[k + 2] = zz.x - z.x;
-      }
-      finite = fx16::fix_matrix<true>(cr, ci, ar, ai, ea);
-    }
+    const bool finite = unpack16(z1, z2, ar, ai, ea, smem_raw, lane);
     bool dk = false;
     int nsw = 0;
     fx16::Result res = fx16::kProduct;
     if (finite) {
-      fx16::add_adjoint<true>(ar, ai, smem_raw, lane);  // 4 C_k, exactly Hermitian
       ea -= 2;
-      fx16::normalise<true>(ar, ai, ea);
       res = fx16::project<true>(ar, ai, ea, v, warm && vstore, smem_raw, lane, &dk, &nsw);
     } else if (!warm) {  // nothing to diagonalise: the store starts from V = I
       fx16::identity_vectors<true>(v, lane);
@@ -731,6 +736,34 @@ __global__ void __launch_bounds__(GroupShape<D>::NT * GroupShape<D>::GPC, GroupS
   }
 }
 
+
+// lmin(C_k) for D = 16: fixed point, one warp a wavevector (ve_fx16.cuh).
+__global__ void __launch_bounds__(32, 16)
+    k_xeig16(const double2* spec, const int* __restrict__ canon, const int ncanon, const FftPlan p, double* lmin) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x;
+  for (int j = blockIdx.x; j < ncanon; j += gridDim.x) {
+    const int s = canon[j], s2 = partner_slot(p, s);
+    fx16::Frag ar, ai;
+    int ea;
+    double w = NAN;
+    if (unpack16(spec + (long)s * 128, spec + (long)s2 * 128, ar, ai, ea, smem_raw, lane))
+      w = fx16::lowest<true>(ar, ai, ea - 2, smem_raw, lane);
+    if (lane == 0) lmin[j] = w;
+    __syncwarp();
+  }
+}
+
+cudaError_t launch_xeig16(const FftPlan& p, const double2* spec, const int* canon, double* lmin, cudaStream_t s) {
+  const size_t smem = fx16::Smem<true>::bytes + fx16::Smem<true>::vectors;
+  static unsigned long long mask = 0;
+  cudaError_t e = smem_once(k_xeig16, smem, mask);
+  if (e != cudaSuccess) return e;
+  const int nc = fft_ncanon(p);
+  const long res = resident_grid((const void*)k_xeig16, 32, smem);
+  k_xeig16<<<(unsigned)(nc < res ? nc : res), 32, smem, s>>>(spec, canon, nc, p, lmin);
+  return cudaGetLastError();
+}
 
 template <int D, typename T>
 cudaError_t launch_xproj_t(const FftPlan& p, double2* spec, const int* canon, void* vstore,
@@ -1201,7 +1234,7 @@ cudaError_t launch_xeig(const FftPlan& p, const double2* spec, const int* canon,
                         cudaStream_t s, unsigned char* gws) {
   switch (p.D) {
     case 4: return launch_xeig_t<4>(p, spec, canon, lmin, s, gws);
-    case 16: return launch_xeig_t<16>(p, spec, canon, lmin, s, gws);
+    case 16: return launch_xeig16(p, spec, canon, lmin, s);
     case 64: return launch_xeig_t<64>(p, spec, canon, lmin, s, gws);
     case 256: return launch_xeig_t<256>(p, spec, canon, lmin, s, gws);
     default: return cudaErrorInvalidValue;

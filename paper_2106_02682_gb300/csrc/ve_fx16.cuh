@@ -49,8 +49,8 @@ using Frag = long long[8];  // one real 16 x 16 matrix, A-fragment layout
 template <bool CPLX>
 struct Smem {
   static constexpr size_t region = (CPLX ? 2 : 1) * (size_t)kD * 512;
-  static constexpr size_t lam = 2 * region;  // 16 float32 eigenvalues
-  static constexpr size_t bytes = lam + 64;
+  static constexpr size_t lam = 2 * region;  // 16 float32 eigenvalues; (EIG) 16 low parts of them
+  static constexpr size_t bytes = lam + 128;
   static constexpr size_t vectors = (CPLX ? 2 : 1) * 256 * 8;  // an eigenvector store of 8-byte words
   static_assert((CPLX ? 2 : 1) * 16 * kLd * 8 <= region && (CPLX ? 4 : 2) * 16 * kLd * 4 <= region, "regions");
 };
@@ -320,10 +320,14 @@ struct Off {
 // redundantly, passed on by shuffles) and its own indices, so a round is two warp barriers.
 // Stops when off(A) <= 1e-10 ||A|| or when the float64 first-order rule holds with a margin of 4 on
 // this matrix, after min_sw sweeps at least.  Returns the sweeps.
+// EIG (eigenvalues): until off(A) has fallen by 1e7 (what float32 angles can give), and the diagonal
+// is held as float32 pairs (low parts in dl): differences of nearly equal eigenvalues decide the angles there, and float32 alone would leave
+// 1e-8 of them on the off-diagonal however often the cycle ran (a projection does not care about
+// the basis within one sign).
 __device__ __forceinline__ int next15(int a) { return a == 14 ? 0 : a + 1; }
 
-template <bool CPLX>
-__device__ int jacobi(float* Ar, float* Ai, float* Qr, float* Qi, int lane, int min_sw, int max_sw) {
+template <bool CPLX, bool EIG>
+__device__ int jacobi(float* Ar, float* Ai, float* Qr, float* Qi, float* dl, int lane, int min_sw, int max_sw) {
   constexpr int LD = kLd;
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
@@ -335,9 +339,10 @@ __device__ int jacobi(float* Ar, float* Ai, float* Qr, float* Qi, int lane, int 
   int k1 = 0, k2 = 0;
   if (lane < 28) rr_pair(8, lane >> 2, lane & 3, k1, k2);
   const int k = lane & 7;
+  [[maybe_unused]] float start = 0.f;
   int sw = 0;
   for (; sw < max_sw; ++sw) {
-    if (sw >= min_sw) {
+    if (EIG || sw >= min_sw) {
       Off f;
       const int j = lane & 15;
       const float lj = Ar[j * LD + j];
@@ -347,7 +352,12 @@ __device__ int jacobi(float* Ar, float* Ai, float* Qr, float* Qi, int lane, int 
         f.add(i, j, Ar[i * LD + j], CPLX ? Ai[i * LD + j] : 0.f, Ar[i * LD + i], lj);
       }
       f.reduce();
-      if (f.off <= 1e-20f * f.nrm2() || f.first_order(4.f)) break;
+      if constexpr (EIG) {
+        if (sw == 0) start = f.off;
+        else if (f.off <= 1e-14f * start) break;
+      } else if (f.off <= 1e-20f * f.nrm2() || f.first_order(4.f)) {
+        break;
+      }
     }
     // indices of the pair this lane rotates and of its block's two pairs, advanced every round
     int a = k == 0 ? 15 : k, b = k == 0 ? 0 : 15 - k;
@@ -364,11 +374,28 @@ __device__ int jacobi(float* Ar, float* Ai, float* Qr, float* Qi, int lane, int 
       } else {
         mag = br;
       }
-      sym_schur2<float>(app, aqq, mag, c, s, t);
+      float npp, nqq, lpp = 0.f, lqq = 0.f;
+      if constexpr (EIG) {
+        const float dp = dl[p], dq = dl[q];
+        sym_schur2<float>(0.f, (aqq - app) + (dq - dp), mag, c, s, t);
+        float e;
+        two_sum(app, -t * mag, npp, e);
+        fast_two_sum(npp, dp + e, npp, lpp);
+        two_sum(aqq, t * mag, nqq, e);
+        fast_two_sum(nqq, dq + e, nqq, lqq);
+      } else {
+        sym_schur2<float>(app, aqq, mag, c, s, t);
+        npp = app - t * mag;
+        nqq = aqq + t * mag;
+      }
       __syncwarp();
       if (lane < 8) {
-        Ar[p * LD + p] = app - t * mag;
-        Ar[q * LD + q] = aqq + t * mag;
+        Ar[p * LD + p] = npp;
+        Ar[q * LD + q] = nqq;
+        if constexpr (EIG) {
+          dl[p] = lpp;
+          dl[q] = lqq;
+        }
         Ar[p * LD + q] = 0.f;
         Ar[q * LD + p] = 0.f;
         if constexpr (CPLX) {
@@ -502,8 +529,9 @@ __device__ __forceinline__ void identity_vectors(long long* v, int lane) {
   }
 }
 
-// V <- the orthonormal factor of V Q in the store; Q: float32 rotations in region 0.
-template <bool CPLX>
+// V <- the orthonormal factor of V Q in the store; Q: float32 rotations in region 0, of which NQ digits
+// are used (four leave ~1e-11 on the off-diagonal of A, six 1e-16).
+template <bool CPLX, int NQ>
 __device__ void update_vectors(long long* v, const float* Qr, const float* Qi, unsigned char* s0, int lane) {
   uint2* f0 = reinterpret_cast<uint2*>(s0);
   Frag xr, xi;
@@ -515,19 +543,19 @@ __device__ void update_vectors(long long* v, const float* Qr, const float* Qi, u
       xr[k] = unit_fix(Qr[o]);
       if constexpr (CPLX) xi[k] = unit_fix(Qi[o]);
     }
-    uint32_t q[4][4], dr[kD][4], di[kD][4];
+    uint32_t q[NQ][4], dr[kD][4], di[kD][4];
     __syncwarp();
-    digits<4>(xr, q);
-    put<4>(q, f0, lane);
+    digits<NQ>(xr, q);
+    put<NQ>(q, f0, lane);
     if constexpr (CPLX) {
-      digits<4>(xi, q);
-      put<4>(q, f0 + 4 * 64, lane);
+      digits<NQ>(xi, q);
+      put<NQ>(q, f0 + NQ * 64, lane);
     }
     load_vectors<CPLX>(v, false, xr, xi, lane);
     digits<kD>(xr, dr);
     if constexpr (CPLX) digits<kD>(xi, di);
     __syncwarp();
-    product<kD, 4, 6, CPLX, 1, 1>(dr, di, f0, xr, xi, lane);
+    product<kD, NQ, 6, CPLX, 1, 1>(dr, di, f0, xr, xi, lane);
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       xr[k] = (xr[k] + 4) >> 3;
@@ -608,7 +636,8 @@ __device__ void update_vectors(long long* v, const float* Qr, const float* Qi, u
   }
 }
 
-enum Result { kProduct, kSame, kZero };  // Y is in the fragments; Y = C; Y = 0
+// Y is in the fragments; Y = C; Y = 0; (EIG) A = V^H C V is in the fragments
+enum Result { kProduct, kSame, kZero, kDiagonal };
 
 // A matrix as fixed point, |X| < 2^53, in the fragment layout.  false when an entry is not finite.
 template <bool CPLX>
@@ -648,9 +677,11 @@ __device__ __forceinline__ void add_adjoint(Frag& r, Frag& i, unsigned char* s0,
 // final ones on return.  *dk: the first-order reconstruction ended
 // it.  *nsw: the float32 Jacobi sweeps taken.  A definite C (found so by the first-order rule)
 // needs no reconstruction: kSame or kZero.
-template <bool CPLX>
+// EIG: no projection; the cycle goes on to the exact rule and leaves A = V^H C V, diagonal but for
+// *off2 = ||E||_F^2 (in units of 2^(2 (53 + ea))).
+template <bool CPLX, bool EIG = false>
 __device__ Result project(Frag& ar, Frag& ai, int& ea, long long* v, bool warm, unsigned char* sm, int lane, bool* dk,
-                          int* nsw) {
+                          int* nsw, float* off2 = nullptr) {
   unsigned char* s0 = sm;
   uint2* f0 = reinterpret_cast<uint2*>(s0);
   uint2* f1 = reinterpret_cast<uint2*>(sm + Smem<CPLX>::region);
@@ -718,12 +749,18 @@ __device__ Result project(Frag& ar, Frag& ai, int& ea, long long* v, bool warm, 
       f.add(i, j, xf[k], yf[k], lam[i], lam[j]);
     }
     f.reduce();
-    *dk = f.first_order(1.f);
+    if constexpr (EIG) {
+      if (f.off <= 3.1554436e-30f * f.nrm2() || cyc == kMaxCycles) {
+        *off2 = f.off;
+        return kDiagonal;
+      }
+    }
+    *dk = !EIG && f.first_order(1.f);
     if (*dk) {
       const unsigned neg = __ballot_sync(0xffffffffu, lam[lane & 15] < 0.f);
       if (neg == 0u || neg == 0xffffffffu) return neg ? kZero : kSame;
     }
-    if (*dk || f.off <= 3.1554436e-30f * f.nrm2() /* (n u)^2 */ || cyc == kMaxCycles) {
+    if (!EIG && (*dk || f.off <= 3.1554436e-30f * f.nrm2() /* (n u)^2 */ || cyc == kMaxCycles)) {
       // M = f(Lambda) + L o E (dk_weight), conjugated, into region 1
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
@@ -758,6 +795,7 @@ __device__ Result project(Frag& ar, Frag& ai, int& ea, long long* v, bool warm, 
       if (i <= j) {
         Jr[i * kLd + j] = xf[k];
         Jr[j * kLd + i] = xf[k];
+        if (EIG && i == j) lam[16 + i] = unit_float(ar[k] - unit_fix(xf[k]));
         if constexpr (CPLX) {
           Ji[i * kLd + j] = i == j ? 0.f : yf[k];
           Ji[j * kLd + i] = i == j ? 0.f : -yf[k];
@@ -765,8 +803,8 @@ __device__ Result project(Frag& ar, Frag& ai, int& ea, long long* v, bool warm, 
       }
     }
     __syncwarp();
-    *nsw += jacobi<CPLX>(Jr, Ji, Qr, Qi, lane, 1, 10);
-    update_vectors<CPLX>(v, Qr, Qi, s0, lane);
+    *nsw += jacobi<CPLX, EIG>(Jr, Ji, Qr, Qi, lam + 16, lane, 1, 10);
+    update_vectors<CPLX, EIG ? kD : 4>(v, Qr, Qi, s0, lane);
   }
   // Y = (conj(Y^T) + Y^T's transpose) / 2
   if constexpr (CPLX) {
@@ -776,6 +814,27 @@ __device__ Result project(Frag& ar, Frag& ai, int& ea, long long* v, bool warm, 
   add_adjoint<CPLX>(ar, ai, s0, lane);
   ea -= 1;
   return kProduct;
+}
+
+// A lower bound on the smallest eigenvalue of C (as in project) by one warp: the smallest diagonal
+// entry of A = V^H C V less ||E||_F (Weyl), whether or not the cycle converged.  `sm` holds Smem and
+// Smem::vectors bytes after it.
+template <bool CPLX>
+__device__ double lowest(Frag& ar, Frag& ai, int ea, unsigned char* sm, int lane) {
+  bool dk;
+  int nsw;
+  float off2 = 0.f;
+  project<CPLX, true>(ar, ai, ea, reinterpret_cast<long long*>(sm + Smem<CPLX>::bytes), false, sm, lane, &dk, &nsw,
+                      &off2);
+  double w = INFINITY;
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    if (frag_row(k, lane) == frag_col(k, lane)) w = nan_min(w, word(ar[k], ea));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) w = nan_min(w, shfl_xor(w, o));
+  __syncwarp();
+  // the sum was taken in float32: rounded up by more than its error
+  return w - 9007199254740992.0 * (double)(sqrtf(off2) * 1.0001f) * word(1, ea);
 }
 
 }  // namespace fx16
