@@ -416,6 +416,10 @@ __device__ int jacobi_sym(T* A, T* V, T* cs, T* red, int tid, bool* dk = nullptr
                           int max_sw = JacobiTol<T>::max_sweeps) {
   static_assert(n == 2 || n % 4 == 0, "the block ordering pairs n / 2 indices");
   constexpr int H = n / 2;
+  // threads that add up the norms: 256 of the 512 a 64 x 64 matrix may have, so that the sums (and
+  // with them the sweep a float32 solve stops at) do not depend on the group's width
+  constexpr int RS = n == 64 && NT > 256 ? 256 : NT;
+  const int rt = tid < RS ? tid : n * n;
   // blocks (GB) and eigenvector rows (GV) a thread loads before it stores any: a matrix staged
   // in global memory (n > 64) needs several loads in flight per thread; every block and row of a
   // round is disjoint from the others, so the reordering changes no result (GV = 8 measured
@@ -425,7 +429,7 @@ __device__ int jacobi_sym(T* A, T* V, T* cs, T* red, int tid, bool* dk = nullptr
   // two-sided update (see below); float64 keeps the symmetric form, its pipe is the bound
   constexpr bool ROWS = n > 64 && !std::is_same<T, double>::value;
   T nrm = T(0);
-  for (int e = tid; e < n * n; e += NT) {
+  for (int e = rt; e < n * n; e += RS) {
     const T a = A[(e / n) * LD + (e % n)];
     nrm += a * a;
   }
@@ -435,12 +439,27 @@ __device__ int jacobi_sym(T* A, T* V, T* cs, T* red, int tid, bool* dk = nullptr
     for (int e = tid; e < n * n; e += NT) V[(e / n) * LD + (e % n)] = (e / n == e % n) ? T(1) : T(0);
   }
   gsync<NT>();
+  // the 2 x 2 blocks (k1, k2), k1 < k2, of a thread that has at most four: row by row, so that a
+  // warp's blocks lie along a row (the circle ordering's k1 + k2 is constant along a run, which put
+  // a run of 16 lanes on one bank: the 64 x 64 float32 projection, 600 -> 430 us)
+  constexpr int NBLK = H * (H - 1) / 2, NOWN = (NBLK + NT - 1) / NT;
+  constexpr bool OWN = NBLK >= 1 && NOWN <= 4;
+  int own1[OWN ? NOWN : 1] = {}, own2[OWN ? NOWN : 1] = {};
+  if constexpr (OWN) {
+#pragma unroll
+    for (int u = 0; u < NOWN; ++u) {
+      if (tid + u * NT < NBLK) {
+        tri_index(H - 1, tid + u * NT, own1[u], own2[u]);
+        ++own2[u];
+      }
+    }
+  }
   if constexpr (DK) *dk = false;
   T off_last = T(0);
   int sweep = 0;
   for (; sweep < max_sw; ++sweep) {
     T off = T(0);
-    for (int e = tid; e < n * n; e += NT) {
+    for (int e = rt; e < n * n; e += RS) {
       const int i = e / n, j = e % n;
       if (i != j) {
         const T a = A[i * LD + j];
@@ -476,14 +495,21 @@ __device__ int jacobi_sym(T* A, T* V, T* cs, T* red, int tid, bool* dk = nullptr
         // the blocks (k1, k2), k1 < k2 -- enumerated as the pairs of a circle ordering of the
         // H pair indices -- and their transposes (k2, k1)
         constexpr int NB = H * (H - 1) / 2;
-        for (int b0 = tid; b0 < NB; b0 += GB * NT) {
+#pragma unroll(OWN ? NOWN : 1)
+        for (int it = 0; it < (NB + GB * NT - 1) / (GB * NT); ++it) {
+          const int b0 = tid + it * GB * NT;
           int k1[GB], k2[GB], p1[GB], q1[GB], p2[GB], q2[GB];
           T m11[GB], m12[GB], m21[GB], m22[GB];
 #pragma unroll
           for (int g = 0; g < GB; ++g) {
             const int b = b0 + g * NT;
             if (b < NB) {
-              rr_pair(H, b / (H / 2), b % (H / 2), k1[g], k2[g]);
+              if constexpr (OWN) {
+                k1[g] = own1[it];
+                k2[g] = own2[it];
+              } else {
+                rr_pair(H, b / (H / 2), b % (H / 2), k1[g], k2[g]);
+              }
               rr_pair(n, r, k1[g], p1[g], q1[g]);
               rr_pair(n, r, k2[g], p2[g], q2[g]);
               m11[g] = A[p1[g] * LD + p2[g]];
@@ -603,10 +629,12 @@ __device__ int jacobi_herm(T* Ar, T* Ai, T* Vr, T* Vi, T* cs, T* red, int tid, b
                            int max_sw = JacobiTol<T>::max_sweeps) {
   static_assert(n % 4 == 0, "the block ordering pairs n / 2 indices");
   constexpr int H = n / 2;
+  constexpr int RS = n == 64 && NT > 256 ? 256 : NT;  // as in jacobi_sym
+  const int rt = tid < RS ? tid : n * n;
   constexpr int GB = n > 64 ? 2 : 1, GV = n > 64 ? 2 : 1;  // as in jacobi_sym (measured)
   constexpr bool ROWS = n > 64 && !std::is_same<T, double>::value;
   T nrm = T(0);
-  for (int e = tid; e < n * n; e += NT) {
+  for (int e = rt; e < n * n; e += RS) {
     const int o = (e / n) * LD + (e % n);
     nrm += Ar[o] * Ar[o] + Ai[o] * Ai[o];
   }
@@ -620,12 +648,25 @@ __device__ int jacobi_herm(T* Ar, T* Ai, T* Vr, T* Vi, T* cs, T* red, int tid, b
     }
   }
   gsync<NT>();
+  // the blocks (k1, k2) of a thread that has at most four, as in jacobi_sym
+  constexpr int NBLK = H * (H - 1) / 2, NOWN = (NBLK + NT - 1) / NT;
+  constexpr bool OWN = NBLK >= 1 && NOWN <= 4;
+  int own1[OWN ? NOWN : 1] = {}, own2[OWN ? NOWN : 1] = {};
+  if constexpr (OWN) {
+#pragma unroll
+    for (int u = 0; u < NOWN; ++u) {
+      if (tid + u * NT < NBLK) {
+        tri_index(H - 1, tid + u * NT, own1[u], own2[u]);
+        ++own2[u];
+      }
+    }
+  }
   if constexpr (DK) *dk = false;
   T off_last = T(0);
   int sweep = 0;
   for (; sweep < max_sw; ++sweep) {
     T off = T(0);
-    for (int e = tid; e < n * n; e += NT) {
+    for (int e = rt; e < n * n; e += RS) {
       const int i = e / n, j = e % n;
       if (i != j) {
         const int o = i * LD + j;
@@ -669,14 +710,21 @@ __device__ int jacobi_herm(T* Ar, T* Ai, T* Vr, T* Vi, T* cs, T* red, int tid, b
       // the blocks (k1, k2), k1 < k2 (pairs of a circle ordering of the H pair indices), and
       // their conjugate transposes (k2, k1)
       constexpr int NB = H * (H - 1) / 2;
-      for (int b0 = tid; b0 < NB; b0 += GB * NT) {
+#pragma unroll(OWN ? NOWN : 1)
+      for (int it = 0; it < (NB + GB * NT - 1) / (GB * NT); ++it) {
+        const int b0 = tid + it * GB * NT;
         int k1[GB], k2[GB], p1[GB], q1[GB], p2[GB], q2[GB];
         T m11r[GB], m11i[GB], m12r[GB], m12i[GB], m21r[GB], m21i[GB], m22r[GB], m22i[GB];
 #pragma unroll
         for (int g = 0; g < GB; ++g) {
           const int b = b0 + g * NT;
           if (b < NB) {
-            rr_pair(H, b / (H / 2), b % (H / 2), k1[g], k2[g]);
+            if constexpr (OWN) {
+              k1[g] = own1[it];
+              k2[g] = own2[it];
+            } else {
+              rr_pair(H, b / (H / 2), b % (H / 2), k1[g], k2[g]);
+            }
             rr_pair(n, r, k1[g], p1[g], q1[g]);
             rr_pair(n, r, k2[g], p2[g], q2[g]);
             m11r[g] = Ar[p1[g] * LD + p2[g]];
@@ -958,6 +1006,14 @@ struct GroupShape {
   // resident CTAs per SM the register budget must allow: at most 128 registers a thread
   static constexpr int MINB = (NT == 32) ? 16 : (NT == 256 ? 2 : 1);
 };
+
+// Threads of a solver kernel's group.  A float32 64 x 64 matrix takes 512: the kernel is bound by the
+// latency of its rounds (a CTA a matrix, tens of matrices), which twice the threads halve but for
+// the rotations themselves.
+template <int n, typename T>
+constexpr int group_threads() {
+  return n == 64 && std::is_same<T, float>::value ? 512 : GroupShape<n>::NT;
+}
 
 // m = sqrt(D) for the pair dimension D = m^2 of a cluster of dimension m.
 template <int D>

@@ -301,11 +301,11 @@ __device__ void unpack_block(const V* spec, int s, int s2, int E, T* Ar, T* Ai, 
 }
 
 template <int D, typename T>
-__global__ void __launch_bounds__(GroupShape<D>::NT * GroupShape<D>::GPC, GroupShape<D>::MINB)
+__global__ void __launch_bounds__(group_threads<D, T>() * GroupShape<D>::GPC, D == 64 ? 1 : GroupShape<D>::MINB)
     k_xproj(typename C2<typename SpecOf<T>::R>::type* spec, const int* __restrict__ canon, const int ncanon,
             const FftPlan p, const double invN, T* vstore, const int warm,
             unsigned long long* stats, unsigned char* gws, const long long* iter) {
-  constexpr int NT = GroupShape<D>::NT, LD = GroupShape<D>::LD;
+  constexpr int NT = group_threads<D, T>(), LD = GroupShape<D>::LD;
   constexpr int GPC = GroupShape<D>::GPC;
   // register-tiled warp products (cgemm16) in float32 only: they compute whole 16 x 16 results
   // where the loops below compute triangles, and float64 / double-float issue is the bound there
@@ -769,7 +769,7 @@ template <int D, typename T>
 cudaError_t launch_xproj_t(const FftPlan& p, double2* spec, const int* canon, void* vstore,
                            int warm, cudaStream_t s, unsigned long long* stats,
                            unsigned char* gws, const long long* iter) {
-  constexpr int NT = GroupShape<D>::NT, GPC = GroupShape<D>::GPC;
+  constexpr int NT = group_threads<D, T>(), GPC = GroupShape<D>::GPC;
   constexpr bool G = GroupShape<D>::GLOBAL;
   const size_t smem = G ? 0 : XSmem<D, T>::bytes * GPC;
   if (!G) {

@@ -35,7 +35,7 @@ constexpr bool FX64 = D == 64 && std::is_same<T, double>::value;
 template <int D, typename T>
 struct PairShape {
   static constexpr int m = ClusterDim<D>::m;
-  static constexpr int NT = FX64<D, T> ? fx64::kThreads : GroupShape<D>::NT;
+  static constexpr int NT = FX64<D, T> ? fx64::kThreads : group_threads<D, T>();
   static constexpr int LD = GroupShape<D>::LD;
   static constexpr int GPC = GroupShape<D>::GPC;  // groups per CTA
 };
@@ -59,7 +59,7 @@ struct PairSmem {
 
 // Arithmetic in T (double, or float in the mixed-precision sweep); the state stays float64.
 template <int D, typename T>
-__global__ void __launch_bounds__(PairShape<D, T>::NT * PairShape<D, T>::GPC, FX64<D, T> ? 1 : GroupShape<D>::MINB)
+__global__ void __launch_bounds__(PairShape<D, T>::NT * PairShape<D, T>::GPC, D == 64 ? 1 : GroupShape<D>::MINB)
     k_pair(const PairArgs a) {
   constexpr int m = PairShape<D, T>::m, NT = PairShape<D, T>::NT, LD = PairShape<D, T>::LD;
   constexpr int GPC = PairShape<D, T>::GPC;
