@@ -228,6 +228,7 @@ PairArgs pair_args(ve_handle* h) {
   a.mu = h->opt.mu;
   a.nu = h->opt.nu;
   a.eps = h->opt.eps;
+  a.k = SolveCoef(a.mu, a.nu, a.m);
   a.rho0 = h->rho0;
   a.rt = h->rt;
   a.lam = h->lam;

@@ -334,14 +334,29 @@ __device__ __forceinline__ void unit_phase<df64>(df64 br, df64 bi, df64& mag, df
 // the distance d of the diagonal from zero: ||R||_F <= c ||E||_F^2 / d (c well below 1 over
 // random 16 x 16 tests).  The sweeps may stop once ||E||_F^2 <= n u ||A||_F d -- as accurate as
 // the exact stopping rule -- provided also ||E||_F <= d / 4, so that no eigenvalue can reach
-// zero.  `off` and `nrm` are the squared Frobenius norms of E and A; the test is uniform over
-// the group.
+// zero.  float64 takes the sharper form of the same bound: f is exact on either sign's block, so R
+// vanishes with B, the part of E between diagonal entries of opposite sign, and ||R||_F <= c ||B||_F
+// ||E||_F / d (c <= 0.19, tests/test_fx16.py): the sweeps stop once ||B||_F ||E||_F <= n u ||A||_F d.
+// `off` and `nrm` are the squared Frobenius norms of E and A; the test is uniform over the group.
 template <typename T, int n, int LD, int NT>
-__device__ bool dk_stop(const T* A, T off, T nrm, T* red, int tid) {
+__device__ bool dk_stop(const T* A, const T* Ai, T off, T nrm, T* red, int tid) {
   T d = T(1e30f);
   for (int k = tid; k < n; k += NT) d = nan_min(d, fabs(A[k * LD + k]));
   d = gmin<NT>(d, red);
-  return off * off <= T(JacobiStop<T, n>::rel2) * nrm * d * d && T(16) * off <= d * d;
+  if constexpr (std::is_same<T, double>::value) {
+    if (!(16.0 * off <= d * d)) return false;
+    double cross = 0.0;
+    for (int e = tid; e < n * n; e += NT) {
+      const int i = e / n, j = e % n;
+      if ((A[i * LD + i] < 0.0) == (A[j * LD + j] < 0.0)) continue;
+      cross = fma(A[i * LD + j], A[i * LD + j], cross);
+      if (Ai) cross = fma(Ai[i * LD + j], Ai[i * LD + j], cross);
+    }
+    cross = gsum<NT>(cross, red);
+    return cross * off <= JacobiStop<T, n>::rel2 * nrm * d * d;
+  } else {
+    return off * off <= T(JacobiStop<T, n>::rel2) * nrm * d * d && T(16) * off <= d * d;
+  }
 }
 
 // 1 / x for x > 0 without a float64 divide: power-of-two scaling, float32 seed, two Newton steps.
@@ -470,7 +485,7 @@ __device__ int jacobi_sym(T* A, T* V, T* cs, T* red, int tid, bool* dk = nullptr
     off_last = off;
     if (off <= T(JacobiStop<T, n>::rel2) * nrm) break;
     if constexpr (DK) {
-      if (dk_stop<T, n, LD, NT>(A, off, nrm, red, tid)) {
+      if (dk_stop<T, n, LD, NT>(A, nullptr, off, nrm, red, tid)) {
         *dk = true;
         break;
       }
@@ -677,7 +692,7 @@ __device__ int jacobi_herm(T* Ar, T* Ai, T* Vr, T* Vi, T* cs, T* red, int tid, b
     off_last = off;
     if (off <= T(JacobiStop<T, n>::rel2) * nrm) break;
     if constexpr (DK) {
-      if (dk_stop<T, n, LD, NT>(Ar, off, nrm, red, tid)) {
+      if (dk_stop<T, n, LD, NT>(Ar, Ai, off, nrm, red, tid)) {
         *dk = true;
         break;
       }

@@ -46,6 +46,7 @@ struct GenArgs {
   int N, m, D, n, L;
   long K;
   double mu, nu, eps;
+  SolveCoef k;
   double* rho;          // N m^2
   double* rt;           // K D^2  rho~
   double* lam;          // K D^2  Lambda
@@ -121,9 +122,7 @@ __global__ void __launch_bounds__(kPairThreads<D>, D == 64 ? 1 : GroupShape<D>::
   T* red = reinterpret_cast<T*>(smem_raw + S::RED);
 
   const T mu = a.mu, nu = a.nu, eps = a.eps;
-  const T alpha = nu * m;
-  const T c0 = T(1) / mu, c1 = T(1) / (mu + alpha), c2 = T(1) / (mu + T(2) * alpha);
-  const T imu = T(1) / mu;
+  const T c0 = a.k.c0, c1 = a.k.c1, c2 = a.k.c2, imu = c0;
   const size_t n = (size_t)a.n;
 
   for (long p = blockIdx.x; p < a.K; p += gridDim.x) {
@@ -675,6 +674,7 @@ GenArgs gen_args(ve_general* h) {
   a.mu = h->opt.mu;
   a.nu = h->opt.nu;
   a.eps = h->opt.eps;
+  a.k = SolveCoef(a.mu, a.nu, a.m);
   a.rho = h->rho;
   a.rt = h->rt;
   a.lam = h->lam;

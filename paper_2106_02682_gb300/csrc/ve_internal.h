@@ -39,9 +39,17 @@ __device__ __forceinline__ bool ns_due(const long long* iter) {
   if (sizeof(T) == 4) return true;
   return iter && (*iter % NS_EVERY) == 0;
 }
+// 1 / mu, 1 / (mu + nu m), 1 / (mu + 2 nu m): the closed-form pair update's constants (a float64
+// divide costs a lone warp ~1 us).
+struct SolveCoef {
+  double c0 = 0, c1 = 0, c2 = 0;
+  SolveCoef() = default;
+  SolveCoef(double mu, double nu, int m) : c0(1.0 / mu), c1(1.0 / (mu + nu * m)), c2(1.0 / (mu + 2.0 * (nu * m))) {}
+};
 struct PairArgs {
   int N, P, m, D;
   double mu, nu, eps;
+  SolveCoef k;
   const double* rho0;   // m*m
   double* rt;           // P*D*D   rho~ (read, then overwritten)
   double* lam;          // P*D*D   Lambda

@@ -83,9 +83,18 @@ __global__ void __launch_bounds__(PairShape<D, T>::NT * PairShape<D, T>::GPC, D 
   T* red = reinterpret_cast<T*>(base + S::RED);
 
   const T mu = (T)a.mu, nu = (T)a.nu, eps = (T)a.eps;
-  const T alpha = nu * m;
-  const T c0 = T(1) / mu, c1 = T(1) / (mu + alpha), c2 = T(1) / (mu + T(2) * alpha);
-  const T imu = T(1) / mu;
+  T c0, c1, c2;
+  if constexpr (std::is_same<T, double>::value) {
+    c0 = a.k.c0;
+    c1 = a.k.c1;
+    c2 = a.k.c2;
+  } else {
+    const T alpha = nu * m;
+    c0 = T(1) / mu;
+    c1 = T(1) / (mu + alpha);
+    c2 = T(1) / (mu + T(2) * alpha);
+  }
+  const T imu = c0;
 
   for (long it = (long)blockIdx.x * GPC + g; it < a.Pc; it += (long)gridDim.x * GPC) {
     const long p = a.pidx ? a.pidx[it] : it;
@@ -372,8 +381,7 @@ struct Pair16Smem {
   static constexpr size_t bytes = fx + fx16::Smem<false>::bytes;
 };
 
-__global__ void __launch_bounds__(32, 16) k_pair16(const PairArgs a, const double c0, const double e1, const double e2,
-                                                   const double imu) {
+__global__ void __launch_bounds__(32, 16) k_pair16(const PairArgs a, const double c0, const double e1, const double e2) {
   using namespace fx16;
   constexpr int D = 16, m = 4, mm = 16;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -464,7 +472,7 @@ __global__ void __launch_bounds__(32, 16) k_pair16(const PairArgs a, const doubl
     bool dk = false;
     double c[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) c[k] = fma(-imu, lv[k], y[k]);
+    for (int k = 0; k < 8; ++k) c[k] = fma(-c0, lv[k], y[k]);
     const bool finite = fix_matrix<false>(c, c, yq, none, ye);
     if (finite) {
       add_adjoint<false>(yq, none, fx, lane);
@@ -546,12 +554,11 @@ cudaError_t launch_pair16(const PairArgs& a, cudaStream_t s) {
   static unsigned long long mask = 0;
   cudaError_t e = smem_once(k_pair16, Pair16Smem::bytes, mask);
   if (e != cudaSuccess) return e;
-  const double m = 4, alpha = a.nu * m;
-  const double c0 = 1.0 / a.mu, c1 = 1.0 / (a.mu + alpha), c2 = 1.0 / (a.mu + 2.0 * alpha);
   long blocks = resident_grid((const void*)k_pair16, 32, Pair16Smem::bytes);
   if (blocks > a.Pc) blocks = a.Pc;
   if (blocks < 1) blocks = 1;
-  k_pair16<<<(unsigned)blocks, 32, Pair16Smem::bytes, s>>>(a, c0, (c1 - c0) / m, (c0 - 2.0 * c1 + c2) / 16.0, c0);
+  k_pair16<<<(unsigned)blocks, 32, Pair16Smem::bytes, s>>>(a, a.k.c0, (a.k.c1 - a.k.c0) / 4,
+                                                        (a.k.c0 - 2.0 * a.k.c1 + a.k.c2) / 16);
   return cudaGetLastError();
 }
 
