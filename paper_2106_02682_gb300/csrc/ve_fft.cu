@@ -10,9 +10,9 @@
 //
 // Transform.  Each pass is a length-n DFT (n <= 64) along one axis of the slot array viewed as
 // [A][n][B], one CTA per (line, chunk of entries): radix-2 stages in registers when n is a power of
-// two (k_fft_pow2), the direct sum otherwise (k_fft_direct).  A 1-D lattice with N > 64 clusters uses
-// the four-step split N = N1 * N2 with a twiddle between the two passes; the spectrum is then
-// stored digit-reversed (slot c*N2 + e holds k = c + N1*e), which the projection handles through
+// two (k_fft_pow2), the direct sum otherwise (k_fft_fold, in float32 k_fft_direct).  A 1-D lattice
+// with N > 64 clusters uses the four-step split N = N1 * N2 with a twiddle between the two passes;
+// the spectrum is then stored digit-reversed (slot c*N2 + e holds k = c + N1*e), which the projection handles through
 // the partner map k -> -k.  A 2-D lattice takes one pass per axis.  Forward sign e^{-i}, no
 // scaling; the projection kernel applies 1/N.
 #include <math.h>
@@ -198,11 +198,10 @@ __global__ void __launch_bounds__(256) k_fft_pow2(const PassIo<R> io, const FftP
   }
 }
 
-// Any n <= 64: the direct sum in shared memory, with the n twiddles there as well (a float64 table
-// entry rounded at every use would cost two conversions at the float64 rate a term).
-template <typename R>
-__global__ void __launch_bounds__(FFT_THREADS) k_fft_direct(const PassIo<R> io, const FftPass ps, const int EC) {
-  using V = typename C2<R>::type;
+// Any n <= 64 in float32: the direct sum in shared memory, with the n twiddles there as well (a
+// float64 table entry rounded at every use would cost two conversions at the float64 rate a term).
+__global__ void __launch_bounds__(FFT_THREADS) k_fft_direct(const PassIo<float> io, const FftPass ps, const int EC) {
+  using V = float2;
   extern __shared__ __align__(16) unsigned char sraw[];
   V* sbuf = reinterpret_cast<V*>(sraw);
   const int la = blockIdx.x / ps.B, lb = blockIdx.x % ps.B;
@@ -219,7 +218,7 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_direct(const PassIo<R> io, 
   for (int idx = threadIdx.x; idx < n * EC; idx += FFT_THREADS) {
     const int k = idx / EC, e = idx % EC;
     if (e >= ec) continue;
-    V acc = C2<R>::make(R(0), R(0));
+    V acc = make_float2(0.f, 0.f);
     for (int j = 0, jk = 0; j < n; ++j) {
       const V t = cmul_term(Wn[jk], sbuf[j * EC + e]);
       acc.x += t.x;
@@ -228,6 +227,57 @@ __global__ void __launch_bounds__(FFT_THREADS) k_fft_direct(const PassIo<R> io, 
       if (jk >= n) jk -= n;
     }
     io.store(ps, la, lb, k, e0 + e, acc);
+  }
+}
+
+// The direct sum in float64, folded: with a_j = x_j + x_{n-j}, b_j = x_j - x_{n-j} (1 <= j <= h,
+// h = floor((n - 1) / 2)) the sums P = sum_j a_j cos, Q = sum_j b_j sin over t = j k serve X_k and
+// X_{n-k} both, X = x_0 + P -+ i Q (+- x_{n/2}): a quarter of the products, and the float64 pipe bounds
+// the pass.  Measured: 170 clusters = 17 x 10, D = 64, a transform 131 us as plain sums, 39 us here;
+// X step of a 30 x 45 lattice, D = 16, 552 and 239 us.
+__global__ void __launch_bounds__(FFT_THREADS) k_fft_fold(const PassIo<double> io, const FftPass ps, const int EC) {
+  extern __shared__ __align__(16) unsigned char sraw[];
+  const int n = ps.n, h = (n - 1) / 2;
+  double2* x = reinterpret_cast<double2*>(sraw);  // x_0, a_1 .. a_h, (x_{n/2}), b_h .. b_1
+  double2* Wn = x + n * EC;                       // (cos, -+ sin) of 2 pi t / n
+  const int la = blockIdx.x / ps.B, lb = blockIdx.x % ps.B;
+  const int e0 = blockIdx.y * EC;
+  const int ec = min(EC, io.E - e0);
+  for (int t = threadIdx.x; t < n; t += FFT_THREADS) Wn[t] = io.twiddle(io.tw[ps.w_off + t]);
+  for (int idx = threadIdx.x; idx < (n - h) * EC; idx += FFT_THREADS) {
+    const int j = idx / EC, e = idx % EC;
+    if (e >= ec) continue;
+    const double2 u = io.load(ps, la, lb, j, e0 + e);
+    if (j == 0 || j > h) {
+      x[idx] = u;
+    } else {
+      const double2 v = io.load(ps, la, lb, n - j, e0 + e);
+      x[idx] = make_double2(u.x + v.x, u.y + v.y);
+      x[(n - j) * EC + e] = make_double2(u.x - v.x, u.y - v.y);
+    }
+  }
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < (n - h) * EC; idx += FFT_THREADS) {
+    const int k = idx / EC, e = idx % EC;
+    if (e >= ec) continue;
+    double px = x[e].x, py = x[e].y, qx = 0.0, qy = 0.0;
+    if ((n & 1) == 0) {
+      const double2 u = x[(n / 2) * EC + e];
+      px += k & 1 ? -u.x : u.x;
+      py += k & 1 ? -u.y : u.y;
+    }
+    for (int j = 1, jk = k; j <= h; ++j) {
+      const double2 w = Wn[jk], a = x[j * EC + e], b = x[(n - j) * EC + e];
+      px = fma(a.x, w.x, px);
+      py = fma(a.y, w.x, py);
+      qx = fma(b.y, w.y, qx);
+      qy = fma(b.x, w.y, qy);
+      jk += k;
+      if (jk >= n) jk -= n;
+    }
+    // w.y = -+ sin: x_j w = (x c - y w.y) + i (y c + x w.y)
+    io.store(ps, la, lb, k, e0 + e, make_double2(px - qx, py + qy));
+    if (k > 0 && 2 * k < n) io.store(ps, la, lb, n - k, e0 + e, make_double2(px + qx, py - qy));
   }
 }
 
@@ -835,7 +885,9 @@ cudaError_t run_pass_t(const FftPlan& p, const FftPass& ps, int dir, const doubl
     case 16: k_fft_pow2<R, 4><<<grid, threads, smem, s>>>(io, ps, ec); break;
     case 32: k_fft_pow2<R, 5><<<grid, threads, smem, s>>>(io, ps, ec); break;
     case 64: k_fft_pow2<R, 6><<<grid, threads, smem, s>>>(io, ps, ec); break;
-    default: k_fft_direct<R><<<grid, FFT_THREADS, smem + sizeof(V) * ps.n, s>>>(io, ps, ec);
+    default:
+      if constexpr (sizeof(R) == 8) k_fft_fold<<<grid, FFT_THREADS, smem + sizeof(V) * ps.n, s>>>(io, ps, ec);
+      else k_fft_direct<<<grid, FFT_THREADS, smem + sizeof(V) * ps.n, s>>>(io, ps, ec);
   }
   return cudaGetLastError();
 }
