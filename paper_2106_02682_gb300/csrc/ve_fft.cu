@@ -81,6 +81,27 @@ __device__ __forceinline__ V cmul_term(V a, V b) {
   return r;
 }
 
+// sg v for sg = +-1, by the sign bit (inv = all bits set where sg = -1, 0 elsewhere): a multiplication
+// would take the float64 pipe, which bounds the float64 passes
+__device__ __forceinline__ float flip(float v, int inv) { return __int_as_float(__float_as_int(v) ^ (inv & (int)0x80000000)); }
+__device__ __forceinline__ double flip(double v, int inv) {
+  return __hiloint2double(__double2hiint(v) ^ (inv & (int)0x80000000), __double2loint(v));
+}
+
+// (u, b) -> (u + w b, u - w b).  Float64: six fused operations instead of eight, u - w b = 2 u - (u + w b);
+// float32 as the rounding of its products is pinned (cmul).
+__device__ __forceinline__ void butterfly(float2 w, float2& u, float2& b) {
+  const float2 t = cmul(w, b);
+  b = make_float2(u.x - t.x, u.y - t.y);
+  u = make_float2(u.x + t.x, u.y + t.y);
+}
+__device__ __forceinline__ void butterfly(double2 w, double2& u, double2& b) {
+  const double2 a = u;
+  u.x = fma(-w.y, b.y, fma(w.x, b.x, a.x));
+  u.y = fma(w.y, b.x, fma(w.x, b.y, a.y));
+  b = make_double2(fma(2.0, a.x, -u.x), fma(2.0, a.y, -u.y));
+}
+
 __device__ __forceinline__ int bitrev(int j, int logn) { return (int)(__brev((unsigned)j) >> (32 - logn)); }
 
 // tf32 part of a float32 value (the significand bits a tf32 tensor-core operand keeps).
@@ -101,14 +122,14 @@ struct PassIo {
   double* xout;
   const double2* __restrict__ tw;
   int E;
-  R sg;  // +1 forward, -1 inverse
+  int inv;  // 0 forward, -1 inverse
 
   __device__ __forceinline__ V load(const FftPass& ps, int la, int lb, int j, int e) const {
     const long slot = ((long)la * ps.n + j) * ps.B + lb;
     if (xin) return C2<R>::make((R)xin[slot * 2 * E + e], (R)xin[slot * 2 * E + E + e]);
     return cin[slot * E + e];
   }
-  __device__ __forceinline__ V twiddle(double2 wd) const { return C2<R>::make((R)wd.x, sg * (R)wd.y); }
+  __device__ __forceinline__ V twiddle(double2 wd) const { return C2<R>::make((R)wd.x, flip((R)wd.y, inv)); }
   __device__ __forceinline__ void store(const FftPass& ps, int la, int lb, int k, int e, V v) const {
     if (ps.tw_mode) {
       const int other = (ps.tw_mode == 1) ? lb : la;
@@ -128,10 +149,11 @@ struct PassIo {
 // one exchange through shared memory between them (n <= 64 needs at most two groups of stages).  A
 // thread owns up to eight points of one column; EC columns a CTA, lanes along the entries.  The
 // twiddles 1 and -i of the first three stages cost no multiplication (10 of 12 butterflies).
-// Float64: the float64 pipe bounds it (1216 instructions a column of 64 against 1536 with every
-// product); float32: L2 latency and the float64 <-> float32 conversions of the block row.
-// Measured (4096 clusters, D = 16, a transform of two passes): 61 us in float64, 21 us in float32; 74
-// and 33 us with every stage through shared memory.
+// Float64: the float64 pipe bounds it (992 instructions a column of 64, 1216 with t = w b, u +- t);
+// float32: L2 latency and the float64 <-> float32 conversions of the block row.
+// Measured (4096 clusters, D = 16, a transform of two passes): 49 us in float64 (61 us before the fused
+// butterflies and the sign by bits, 74 us with every stage through shared memory), 20 us in float32
+// (33 us through shared memory).
 template <typename R, int L>
 __global__ void __launch_bounds__(256) k_fft_pow2(const PassIo<R> io, const FftPass ps, const int EC) {
   using V = typename C2<R>::type;
@@ -156,10 +178,11 @@ __global__ void __launch_bounds__(256) k_fft_pow2(const PassIo<R> io, const FftP
       if (i0 & half) continue;
       const int j = i0 & (half - 1);
       const V u = x[i0], b = x[i0 + half];
-      V t;
-      if (j == 0) t = b;
-      else if (2 * j == half) t = C2<R>::make(io.sg * b.y, -io.sg * b.x);  // -i b (inverse: i b)
-      else t = cmul(io.twiddle(Wn[j * (n / (2 * half))]), b);
+      if (j != 0 && 2 * j != half) {
+        butterfly(io.twiddle(Wn[j * (n / (2 * half))]), x[i0], x[i0 + half]);
+        continue;
+      }
+      const V t = j == 0 ? b : C2<R>::make(flip(b.y, io.inv), flip(b.x, ~io.inv));  // -i b (inverse: i b)
       x[i0] = C2<R>::make(u.x + t.x, u.y + t.y);
       x[i0 + half] = C2<R>::make(u.x - t.x, u.y - t.y);
     }
@@ -186,9 +209,7 @@ __global__ void __launch_bounds__(256) k_fft_pow2(const PassIo<R> io, const FftP
         for (int i0 = 0; i0 < G; ++i0) {
           if (i0 & half) continue;
           const int j = q + 8 * (i0 & (half - 1));
-          const V u = y[i0], t = cmul(io.twiddle(Wn[j * (n / (16 * half))]), y[i0 + half]);
-          y[i0] = C2<R>::make(u.x + t.x, u.y + t.y);
-          y[i0 + half] = C2<R>::make(u.x - t.x, u.y - t.y);
+          butterfly(io.twiddle(Wn[j * (n / (16 * half))]), y[i0], y[i0 + half]);
         }
       }
 #pragma unroll
@@ -874,7 +895,7 @@ cudaError_t run_pass_t(const FftPlan& p, const FftPass& ps, int dir, const doubl
     while (ec > 8 && lines * ((p.E + ec - 1) / ec) < 304) ec /= 2;
   }
   const PassIo<R> io = {xin, reinterpret_cast<const V*>(cin), reinterpret_cast<V*>(cout), xout, tw, p.E,
-                        dir > 0 ? R(-1) : R(1)};
+                        dir > 0 ? -1 : 0};
   const dim3 grid((unsigned)lines, (unsigned)((p.E + ec - 1) / ec));
   const size_t smem = sizeof(V) * ps.n * ec;  // at most 32 KB (33 with the direct sum's twiddles)
   const int threads = ps.n > 8 ? ec * (ps.n / 8) : ec;
