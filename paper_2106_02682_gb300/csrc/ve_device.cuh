@@ -431,9 +431,10 @@ __device__ int jacobi_sym(T* A, T* V, T* cs, T* red, int tid, bool* dk = nullptr
                           int max_sw = JacobiTol<T>::max_sweeps) {
   static_assert(n == 2 || n % 4 == 0, "the block ordering pairs n / 2 indices");
   constexpr int H = n / 2;
-  // threads that add up the norms: 256 of the 512 a 64 x 64 matrix may have, so that the sums (and
-  // with them the sweep a float32 solve stops at) do not depend on the group's width
-  constexpr int RS = n == 64 && NT > 256 ? 256 : NT;
+  // threads that add up the norms: 256 of the 512 a 64 x 64 matrix may have and one warp for a
+  // 32 x 32 one, so that the sums (and with them the sweep a float32 solve stops at) do not depend
+  // on the group's width
+  constexpr int RS = n == 32 ? 32 : n == 64 && NT > 256 ? 256 : NT;
   const int rt = tid < RS ? tid : n * n;
   // blocks (GB) and eigenvector rows (GV) a thread loads before it stores any: a matrix staged
   // in global memory (n > 64) needs several loads in flight per thread; every block and row of a
@@ -443,6 +444,9 @@ __device__ int jacobi_sym(T* A, T* V, T* cs, T* red, int tid, bool* dk = nullptr
   // a matrix in global memory in float32 / double-float words takes the row-block form of the
   // two-sided update (see below); float64 keeps the symmetric form, its pipe is the bound
   constexpr bool ROWS = n > 64 && !std::is_same<T, double>::value;
+  // the lanes of a warp along the rows of V (one pair, its rotation broadcast): with the odd leading
+  // dimension no two lanes share a bank, and the pair's indices are the same for the warp
+  constexpr bool LANE_ROWS = n == 32 || n == 64;
   T nrm = T(0);
   for (int e = rt; e < n * n; e += RS) {
     const T a = A[(e / n) * LD + (e % n)];
@@ -600,8 +604,8 @@ __device__ int jacobi_sym(T* A, T* V, T* cs, T* red, int tid, bool* dk = nullptr
           for (int g = 0; g < GV; ++g) {
             const int t = t0 + g * NT;
             if (t < n * H) {
-              ix[g] = t / H;
-              kk[g] = t % H;
+              ix[g] = LANE_ROWS ? t % n : t / H;
+              kk[g] = LANE_ROWS ? t / n : t % H;
               rr_pair(n, r, kk[g], pp[g], qq[g]);
               vp[g] = V[ix[g] * LD + pp[g]];
               vq[g] = V[ix[g] * LD + qq[g]];
@@ -644,10 +648,11 @@ __device__ int jacobi_herm(T* Ar, T* Ai, T* Vr, T* Vi, T* cs, T* red, int tid, b
                            int max_sw = JacobiTol<T>::max_sweeps) {
   static_assert(n % 4 == 0, "the block ordering pairs n / 2 indices");
   constexpr int H = n / 2;
-  constexpr int RS = n == 64 && NT > 256 ? 256 : NT;  // as in jacobi_sym
+  constexpr int RS = n == 32 ? 32 : n == 64 && NT > 256 ? 256 : NT;  // as in jacobi_sym
   const int rt = tid < RS ? tid : n * n;
   constexpr int GB = n > 64 ? 2 : 1, GV = n > 64 ? 2 : 1;  // as in jacobi_sym (measured)
   constexpr bool ROWS = n > 64 && !std::is_same<T, double>::value;
+  constexpr bool LANE_ROWS = n == 32 || n == 64;  // as in jacobi_sym
   T nrm = T(0);
   for (int e = rt; e < n * n; e += RS) {
     const int o = (e / n) * LD + (e % n);
@@ -860,8 +865,8 @@ __device__ int jacobi_herm(T* Ar, T* Ai, T* Vr, T* Vi, T* cs, T* red, int tid, b
           for (int g = 0; g < GV; ++g) {
             const int t = t0 + g * NT;
             if (t < n * H) {
-              ix[g] = t / H;
-              kk[g] = t % H;
+              ix[g] = LANE_ROWS ? t % n : t / H;
+              kk[g] = LANE_ROWS ? t / n : t % H;
               rr_pair(n, r, kk[g], pp[g], qq[g]);
               vpr[g] = Vr[ix[g] * LD + pp[g]];
               vpi[g] = Vi[ix[g] * LD + pp[g]];

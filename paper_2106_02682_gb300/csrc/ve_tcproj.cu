@@ -181,19 +181,19 @@ __global__ void __launch_bounds__(kNT, 1)
 
 // ---- block Jacobi: the 256 indices form TC_BJ_NB = 16 blocks of TC_BJ_BS = 16; a round pairs
 // the blocks by the circle ordering (15 rounds a sweep, 8 disjoint pairs a round).  For each pair
-// (I, J) the 32 x 32 principal block A[I u J, I u J] is diagonalised exactly by one warp in shared
+// (I, J) the 32 x 32 principal block A[I u J, I u J] is diagonalised by one CTA in shared
 // memory (k_bj_sub), its eigenvectors U placed in the round's rotation R (R[I u J, I u J] = U,
 // zero elsewhere), and A <- R^H A R, V <- V R are three tensor-core products that touch only
 // R's nonzero blocks (tc_rot256), which are stored compactly (one 32 x 32 block per pair).  A sweep of rounds annihilates every off-diagonal
 // block once; like scalar Jacobi it converges quadratically.
-constexpr int kBS = TC_BJ_BS, kNB = TC_BJ_NB, kSub = 2 * kBS, kSLD = kSub + 1, kSubWarps = 4;
+constexpr int kBS = TC_BJ_BS, kNB = TC_BJ_NB, kSub = 2 * kBS, kSLD = kSub + 1;
+constexpr int kSubNT = 128;
 constexpr int kRc = kN * kSub;  // floats of one plane of a compact rotation (256 rows x 32 K)
 
 template <bool CPLX>
 struct SubShape {
   static constexpr int NMAT = CPLX ? 4 : 2;
-  static constexpr size_t per_warp = sizeof(float) * (NMAT * kSub * kSLD + 2 * kSub + 32);
-  static constexpr size_t bytes = per_warp * kSubWarps;
+  static constexpr size_t bytes = sizeof(float) * (NMAT * kSub * kSLD + 2 * kSub + 32);
 };
 
 __device__ __forceinline__ int kc4i(int r, int k) { return ((k >> 2) * kN + r) * 4 + (k & 3); }
@@ -216,36 +216,42 @@ __global__ void __launch_bounds__(256) k_fro2(const float* __restrict__ A, int n
 // test off^2 <= (n u)^2 ||A||^2 over 120 block pairs of a sweep holds for the matrix when every
 // block meets off^2 <= (256 u)^2 ||A||^2 / 120, i.e. the block test (32 u)^2 nrm with
 // nrm >= (256 / 32)^2 / 120 ||A||^2 ~ 0.5 ||A||^2.
+//
+// Shared-memory accesses and the index arithmetic bound it.  Four warps a block solve: 120 of the 128
+// threads own one 2 x 2 block of a round, and CTAs of one solve each leave no last wave of whole
+// CTAs.  Measured (513 wavevectors, 30 rounds with their rotation products): 29.1 ms with a warp a
+// solve, 27.0 ms here (27.8 with two warps, 28.2 with eight); 512 real pair projections 16.7 and
+// 15.9 ms.
 template <bool CPLX>
-__global__ void __launch_bounds__(32 * kSubWarps)
+__global__ void __launch_bounds__(kSubNT)
     k_bj_sub(const float* __restrict__ A, float* __restrict__ Rt, long count, int round,
              const float* __restrict__ fro2, int max_inner) {
   constexpr int NPL = CPLX ? 4 : 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float* Sr = reinterpret_cast<float*>(smem_raw + w * SubShape<CPLX>::per_warp);
+  const int tid = threadIdx.x;
+  float* Sr = reinterpret_cast<float*>(smem_raw);
   float* Ur = Sr + kSub * kSLD;
   float* Si = CPLX ? Ur + kSub * kSLD : nullptr;
   float* Ui = CPLX ? Si + kSub * kSLD : nullptr;
   float* cs = Sr + SubShape<CPLX>::NMAT * kSub * kSLD;
   float* red = cs + 2 * kSub;
   const long items = count * (kNB / 2);
-  for (long item = (long)blockIdx.x * kSubWarps + w; item < items; item += (long)gridDim.x * kSubWarps) {
+  for (long item = blockIdx.x; item < items; item += gridDim.x) {
     const long b = item / (kNB / 2);
     const int k = (int)(item % (kNB / 2));
     int bp, bq;
     rr_pair(kNB, round, k, bp, bq);
     auto g = [&](int t) { return t < kBS ? bp * kBS + t : bq * kBS + (t - kBS); };
     const float* a = A + (size_t)b * (NPL / 2) * kPl;  // plain: re (, im)
-    for (int e = lane; e < kSub * kSub; e += 32) {
+    for (int e = tid; e < kSub * kSub; e += kSubNT) {
       const int i = e / kSub, j = e % kSub;
       const int o = kc4i(g(i), g(j));
       Sr[i * kSLD + j] = a[o];
       if constexpr (CPLX) Si[i * kSLD + j] = a[kPl + o];
     }
-    __syncwarp();
+    __syncthreads();
     // (S + S^H) / 2
-    for (int e = lane; e < kSub * kSub; e += 32) {
+    for (int e = tid; e < kSub * kSub; e += kSubNT) {
       const int i = e / kSub, j = e % kSub;
       if (i < j) {
         const float v = 0.5f * (Sr[i * kSLD + j] + Sr[j * kSLD + i]);
@@ -260,19 +266,19 @@ __global__ void __launch_bounds__(32 * kSubWarps)
         if constexpr (CPLX) Si[i * kSLD + i] = 0.f;
       }
     }
-    __syncwarp();
+    __syncthreads();
     const float floor2 = 0.5f * fro2[b];
     if constexpr (CPLX)
-      jacobi_herm<float, kSub, kSLD, 32, true>(Sr, Si, Ur, Ui, cs, red, lane, nullptr, nullptr, floor2,
+      jacobi_herm<float, kSub, kSLD, kSubNT, true>(Sr, Si, Ur, Ui, cs, red, tid, nullptr, nullptr, floor2,
                                                max_inner);
     else
-      jacobi_sym<float, kSub, kSLD, 32, true>(Sr, Ur, cs, red, lane, nullptr, nullptr, floor2, max_inner);
+      jacobi_sym<float, kSub, kSLD, kSubNT, true>(Sr, Ur, cs, red, tid, nullptr, nullptr, floor2, max_inner);
     // The round's rotation, compact: per matrix NPL split planes of 256 rows x 32 K (KC4), row
     // 32 k + c and K index a holding U[a][c] (pair-local indices, block bp then block bq): the
     // rotation products read each pair's 32 x 32 block as one box.  A lane writes one 4-index
     // chunk of one row as a float4.
     float* rc = Rt + (size_t)b * NPL * kRc;
-    for (int e = lane; e < kSub * (kSub / 4); e += 32) {
+    for (int e = tid; e < kSub * (kSub / 4); e += kSubNT) {
       const int c = e / (kSub / 4), ch = e % (kSub / 4);  // row 32 k + c, K chunk 4 ch .. + 3
       float ur[4], ui[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -291,7 +297,7 @@ __global__ void __launch_bounds__(32 * kSubWarps)
         *reinterpret_cast<float4*>(rc + 3 * kRc + o) = lo;
       }
     }
-    __syncwarp();
+    __syncthreads();
   }
 }
 
@@ -390,8 +396,7 @@ cudaError_t tc_project256(TcProjWs& w, long count, bool warm, unsigned long long
       attr[w.cplx] = true;
     }
     const long items = count * (kNB / 2);
-    const long ctas = (items + kSubWarps - 1) / kSubWarps;
-    const int sgrid = (int)(ctas < 8L * big_grid() ? ctas : 8L * big_grid());
+    const int sgrid = (int)(items < (1L << 20) ? items : 1L << 20);
     float* fro2 = reinterpret_cast<float*>(w.M);  // M is free until the polish
     k_fro2<<<(unsigned)count, 256, 0, s>>>(A, w.cplx ? 2 : 1, fro2);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -405,9 +410,9 @@ cudaError_t tc_project256(TcProjWs& w, long count, bool warm, unsigned long long
     for (int sw = 0; sw < w.bj_sweeps; ++sw) {
       for (int r = 0; r < kNB - 1; ++r) {
         if (w.cplx)
-          k_bj_sub<true><<<sgrid, 32 * kSubWarps, smem, s>>>(A, w.Qt, count, r, fro2, inner);
+          k_bj_sub<true><<<sgrid, kSubNT, smem, s>>>(A, w.Qt, count, r, fro2, inner);
         else
-          k_bj_sub<false><<<sgrid, 32 * kSubWarps, smem, s>>>(A, w.Qt, count, r, fro2, inner);
+          k_bj_sub<false><<<sgrid, kSubNT, smem, s>>>(A, w.Qt, count, r, fro2, inner);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         // B = A R (kept transposed in Wt); A <- R^H B written as (B^H R)^H; V1 <- V1 R.  All
         // three multiply by the block rotation R on the right (tc_rot256: its nonzero blocks
