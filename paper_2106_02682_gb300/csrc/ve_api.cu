@@ -177,7 +177,7 @@ struct ve_handle {
          *H0 = nullptr, *lmin_pairs = nullptr, *lmin_k = nullptr, *lmin0 = nullptr;
   int *hslot = nullptr, *neg = nullptr, *canon = nullptr;
   int ncanon = 0;
-  // pair offsets tied to their opposite (k_pair, k_dual12): Pc work items
+  // pair offsets tied to their opposite (k_pair, k_dual_status): Pc work items
   int Pc = 0;
   int *pidx = nullptr, *pmir = nullptr, *ptie = nullptr;
   double2 *specA = nullptr, *specB = nullptr, *tw = nullptr;

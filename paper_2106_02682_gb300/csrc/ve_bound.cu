@@ -8,8 +8,8 @@
 //   F[X] >= N lmin(K_0) + sum_delta c(delta) lmin(K_delta),
 //   K_delta = H'_{0,delta} + Lambda1_delta (x) I + I (x) Lambda1_{-delta},
 //   K_0     = H'_0 - sum_delta Lambda1_delta.
-// This file computes lmin(K_delta) for every delta and lmin(K_0) in float64 (values-only
-// Jacobi); the host adds the weights c(delta) and the correction for a slightly indefinite X.
+// This file computes lmin(K_delta) for every delta and lmin(K_0) in float64 (values-only Jacobi;
+// D = 16 in fixed point, ve_fx16.cuh); the host adds the weights c(delta) and the correction for a slightly indefinite X.
 // Each lmin is the smallest diagonal entry of the rotated matrix minus the Frobenius norm of its
 // remaining off-diagonal part, a lower bound by Weyl's inequality whether or not the Jacobi
 // sweeps converged; minima pass a NaN on (nan_min), so a non-finite state cannot certify.

@@ -215,14 +215,6 @@ __global__ void __launch_bounds__(256) k_dense_rayleigh(const double* Vt, const 
   if (lane == 0) lam[i] = s;
 }
 
-__global__ void __launch_bounds__(256) k_dense_min(const double* lam, int n, DenseCtl* ctl) {
-  __shared__ double red[8];
-  double v = INFINITY;
-  for (int k = threadIdx.x; k < n; k += 256) v = nan_min(v, lam[k]);
-  v = gmin<256>(v, red);
-  if (threadIdx.x == 0) ctl->lmin = v;
-}
-
 // A certified lmin from the explicit A = V^T Y V = diag + E (B[i][j] = v_i.w_j, symmetrised):
 // by Weyl's inequality every eigenvalue of A lies within ||E||_2 <= ||E||_F of the sorted
 // diagonal, so lmin(Y) >= min_i a_ii - ||E||_F whether or not the sweeps converged.  A NaN
@@ -380,9 +372,6 @@ int dense_ws_init(DenseWs& w, int n, void* mem, size_t bytes) {
 }
 
 void dense_ws_release(DenseWs& w) {
-  if (w.g0) cudaEventDestroy(w.g0);
-  if (w.g1) cudaEventDestroy(w.g1);
-  w.g0 = w.g1 = nullptr;
   if (w.exec) cudaGraphExecDestroy(w.exec);
   if (w.graph) cudaGraphDestroy(w.graph);
   if (w.hctl) cudaFreeHost(w.hctl);
@@ -445,25 +434,13 @@ cudaError_t dense_eig(DenseWs& w, const double* Y, int mode, cudaStream_t s) {
   e = gemm<false, true>(n, n, n, w.Vt, n, Y, n, w.Wt, n, nullptr, s);
   if (e != cudaSuccess) return e;
   w.launches += 1;
-  if (w.prof && !w.g0) {
-    if ((e = cudaEventCreate(&w.g0)) != cudaSuccess) return e;
-    if ((e = cudaEventCreate(&w.g1)) != cudaSuccess) return e;
-  }
   int sweeps = 0;
   for (; sweeps < JacobiTol<double>::max_sweeps; ++sweeps) {
-    if (w.prof && (e = cudaEventRecord(w.g0, s)) != cudaSuccess) return e;
     if ((e = cudaGraphLaunch(w.exec, s)) != cudaSuccess) return e;
-    if (w.prof && (e = cudaEventRecord(w.g1, s)) != cudaSuccess) return e;
     w.launches += n;
     if ((e = cudaMemcpyAsync(w.hctl, w.ctl, sizeof(DenseCtl), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
       return e;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-    if (w.prof) {
-      float ms = 0.f;
-      if ((e = cudaEventElapsedTime(&ms, w.g0, w.g1)) != cudaSuccess) return e;
-      w.graph_ms += ms;
-      w.graph_rounds += n - 1;
-    }
     if (w.hctl->converged) {
       ++sweeps;
       break;
@@ -508,12 +485,6 @@ cudaError_t dense_reconstruct(DenseWs& w, double* X, cudaStream_t s) {
   const cudaError_t e = gemm<true, false>(n, n, n, w.Vt, n, w.Vt, n, X, n, w.lam, s);
   w.launches += 1;
   return e;
-}
-
-cudaError_t dense_lmin(DenseWs& w, cudaStream_t s) {
-  k_dense_min<<<1, 256, 0, s>>>(w.lam, w.n, w.ctl);
-  w.launches += 1;
-  return cudaGetLastError();
 }
 
 cudaError_t dense_lmin_certified(DenseWs& w, cudaStream_t s) {

@@ -11,7 +11,7 @@ constexpr int DENSE_MAX_N = 1024;  // a round CTA holds 8 entries of each of its
 struct DenseCtl {
   double nrm2;   // ||Y||_F^2
   double off2;   // 2 sum a_pq^2 over the last sweep's rotations
-  double lmin;   // smallest lambda_i (dense_lmin)
+  double lmin;   // lower bound on the smallest eigenvalue (dense_lmin_certified)
   int converged; // the last sweep met the stopping rule
   int sweeps;    // sweeps of the current eigensolve
   int dk;        // explicit check: 0 go on, 1 converged, 2 first-order reconstruction suffices
@@ -37,11 +37,6 @@ struct DenseWs {
   int last_sweeps = 0;
   long total_sweeps = 0;
   long launches = 0;        // kernels launched (graph rounds counted one by one)
-  // profiling: CUDA events around every sweep graph (created on first use when prof is set)
-  bool prof = false;
-  cudaEvent_t g0 = nullptr, g1 = nullptr;
-  double graph_ms = 0.0;    // device time of the profiled sweep graphs
-  long graph_rounds = 0;    // round launches in them
 };
 
 enum { DENSE_COLD = 0, DENSE_WARM = 1 };
@@ -59,8 +54,6 @@ cudaError_t dense_eig(DenseWs& w, const double* Y, int mode, cudaStream_t s);
 // X = V diag(max(lambda, 0)) V^T after dense_eig, or V (f(Lambda) + L o E) V^T when the
 // eigensolve took the first-order stop (X may alias the Y given to dense_eig).
 cudaError_t dense_reconstruct(DenseWs& w, double* X, cudaStream_t s);
-// ctl->lmin = min_i lambda_i after dense_eig.
-cudaError_t dense_lmin(DenseWs& w, cudaStream_t s);
 // ctl->lmin = min_i a_ii - ||offdiag(A)||_F for A = V^T Y V formed from Vt and Wt after
 // dense_eig: a lower bound on lmin(Y) by Weyl's inequality (one GEMM into Bt).
 cudaError_t dense_lmin_certified(DenseWs& w, cudaStream_t s);

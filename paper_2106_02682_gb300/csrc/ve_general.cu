@@ -5,15 +5,16 @@
 //
 // One sweep on the GPU:
 //   k5_pair    one thread group per pair: H'_ij (Eq. (effHam)), the closed-form rho_ij
-//              (Eq. (rhoijUpdate)), rho~_ij = Pi(rho_ij - Lambda_ij / mu) by the warm-started
-//              Jacobi of the Algorithm-6 pair pass (Eq. (rhoijTildeUpdate)), the Lambda update,
+//              (Eq. (rhoijUpdate)), rho~_ij = Pi(rho_ij - Lambda_ij / mu) by the projections of
+//              the Algorithm-6 pair pass (Eq. (rhoijTildeUpdate)): fixed point for D = 16 and 64,
+//              warm-started Jacobi for D = 4 and 256, the Lambda update,
 //              A1 rho, A2 rho, and the off-diagonal blocks of Y = X - eps G (G_ij and G_ji =
 //              G_ij^T, Sec. 2.2);
 //   k5_rho     one CTA per cluster: Eq. (rhoiUpdate) over the pairs on either side with the
 //              trace shift, and the diagonal block Y_ii = X_ii - eps G_00[rho_i];
 //   k5_dual    Lambda1 / Lambda2 updates with the new rho_i;
 //   k5_status  energy per spin, Eq. (feasErr), residual (fixed-order sums);
-//   X = Pi(Y)  the whole-GPU dense eigensolver of ve_dense.cu (warm-started).
+//   X = Pi(Y)  the whole-GPU matrix sign iteration of ve_fxsign.cu.
 // The X step takes the sign X - eps G: the ascent direction of the dual function, the only
 // sign whose fixed point meets the optimality conditions (the paper prints X + eps G).
 #include <cuda_runtime.h>
