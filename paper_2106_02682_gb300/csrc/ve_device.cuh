@@ -103,8 +103,11 @@ __device__ __forceinline__ void rr_pair(int n, int r, int k, int& p, int& q) {
     a = n - 1;
     b = r;
   } else {
-    a = (r + k) % (n - 1);
-    b = (r - k + n - 1) % (n - 1);
+    // both below 2 (n - 1), reduced by one subtraction (x - (n - 1) wraps to a large number where
+    // x < n - 1); a remainder by a constant takes four instructions, four times a block and round
+    const unsigned x = r + k, y = r - k + n - 1, m = n - 1;
+    a = (int)min(x, x - m);
+    b = (int)min(y, y - m);
   }
   p = a < b ? a : b;
   q = a < b ? b : a;
