@@ -476,6 +476,32 @@ __device__ int jacobi_sym(T* A, T* V, T* cs, T* red, int tid, bool* dk = nullptr
       }
     }
   }
+  // the rotations of round r + 1 by the first warp while the others update V for round r: they are a
+  // serial chain of divides and square roots on H lanes (64 x 64 float32, 25 matrices: 258 -> 243 us
+  // real, 384 -> 357 us complex)
+  constexpr bool PIPE = VEC && LANE_ROWS && NT > 32;
+  T* cs2 = cs;
+  if constexpr (PIPE) {
+    __shared__ T other[n];
+    cs2 = other;
+  }
+  // the rotation of each pair, and the pair's own 2x2 block made diagonal
+  auto rotations = [&](int r, T* rot) {
+    for (int k = tid; k < H; k += NT) {
+      int p, q;
+      rr_pair(n, r, k, p, q);
+      const T app = A[p * LD + p], aqq = A[q * LD + q], apq = A[p * LD + q];
+      T c, s, t;
+      sym_schur2<T>(app, aqq, apq, c, s, t);
+      rot[k] = c;
+      rot[H + k] = s;
+      A[p * LD + p] = app - t * apq;
+      A[q * LD + q] = aqq + t * apq;
+      A[p * LD + q] = T(0);
+      A[q * LD + p] = T(0);
+    }
+  };
+  T* const cs1 = cs;
   if constexpr (DK) *dk = false;
   T off_last = T(0);
   int sweep = 0;
@@ -498,21 +524,11 @@ __device__ int jacobi_sym(T* A, T* V, T* cs, T* red, int tid, bool* dk = nullptr
       }
     }
     for (int r = 0; r < n - 1; ++r) {
-      // the rotation of each pair, and the pair's own 2x2 block made diagonal
-      for (int k = tid; k < H; k += NT) {
-        int p, q;
-        rr_pair(n, r, k, p, q);
-        const T app = A[p * LD + p], aqq = A[q * LD + q], apq = A[p * LD + q];
-        T c, s, t;
-        sym_schur2<T>(app, aqq, apq, c, s, t);
-        cs[k] = c;
-        cs[H + k] = s;
-        A[p * LD + p] = app - t * apq;
-        A[q * LD + q] = aqq + t * apq;
-        A[p * LD + q] = T(0);
-        A[q * LD + p] = T(0);
+      cs = (r & 1) ? cs2 : cs1;
+      if (!PIPE || r == 0) {
+        rotations(r, cs);
+        gsync<NT>();
       }
-      gsync<NT>();
       if constexpr (H >= 2 && !ROWS) {
         // the blocks (k1, k2), k1 < k2 -- enumerated as the pairs of a circle ordering of the
         // H pair indices -- and their transposes (k2, k1)
@@ -599,13 +615,18 @@ __device__ int jacobi_sym(T* A, T* V, T* cs, T* red, int tid, bool* dk = nullptr
           }
         }
       }
+      if constexpr (PIPE) {
+        gsync<NT>();
+        if (r + 1 < n - 1) rotations(r + 1, (r & 1) ? cs1 : cs2);
+      }
       if constexpr (VEC) {
-        for (int t0 = tid; t0 < n * H; t0 += GV * NT) {
+        constexpr int VT = PIPE ? NT - 32 : NT;
+        for (int t0 = !PIPE ? tid : tid < 32 ? n * H : tid - 32; t0 < n * H; t0 += GV * VT) {
           int ix[GV], kk[GV], pp[GV], qq[GV];
           T vp[GV], vq[GV];
 #pragma unroll
           for (int g = 0; g < GV; ++g) {
-            const int t = t0 + g * NT;
+            const int t = t0 + g * VT;
             if (t < n * H) {
               ix[g] = LANE_ROWS ? t % n : t / H;
               kk[g] = LANE_ROWS ? t / n : t % H;
@@ -616,7 +637,7 @@ __device__ int jacobi_sym(T* A, T* V, T* cs, T* red, int tid, bool* dk = nullptr
           }
 #pragma unroll
           for (int g = 0; g < GV; ++g) {
-            if (t0 + g * NT < n * H) {
+            if (t0 + g * VT < n * H) {
               const T c = cs[kk[g]], s = cs[H + kk[g]];
               V[ix[g] * LD + pp[g]] = c * vp[g] - s * vq[g];
               V[ix[g] * LD + qq[g]] = s * vp[g] + c * vq[g];
@@ -684,6 +705,37 @@ __device__ int jacobi_herm(T* Ar, T* Ai, T* Vr, T* Vi, T* cs, T* red, int tid, b
       }
     }
   }
+  constexpr bool PIPE = VEC && LANE_ROWS && NT > 32;  // as in jacobi_sym
+  T* cs2 = cs;
+  if constexpr (PIPE) {
+    __shared__ T other[2 * n];
+    cs2 = other;
+  }
+  // the rotation of each pair, and the pair's own 2x2 block made (real) diagonal
+  auto rotations = [&](int r, T* rot) {
+    for (int k = tid; k < H; k += NT) {
+      int p, q;
+      rr_pair(n, r, k, p, q);
+      const T app = Ar[p * LD + p], aqq = Ar[q * LD + q];
+      const T br = Ar[p * LD + q], bi = Ai[p * LD + q];
+      T c, s, t, mag = T(0), wr = T(1), wi = T(0);
+      if (br != T(0) || bi != T(0)) unit_phase<T>(br, bi, mag, wr, wi);
+      sym_schur2<T>(app, aqq, mag, c, s, t);
+      rot[k] = c;
+      rot[H + k] = s;
+      rot[2 * H + k] = wr;
+      rot[3 * H + k] = wi;
+      Ar[p * LD + p] = app - t * mag;
+      Ar[q * LD + q] = aqq + t * mag;
+      Ai[p * LD + p] = T(0);
+      Ai[q * LD + q] = T(0);
+      Ar[p * LD + q] = T(0);
+      Ai[p * LD + q] = T(0);
+      Ar[q * LD + p] = T(0);
+      Ai[q * LD + p] = T(0);
+    }
+  };
+  T* const cs1 = cs;
   if constexpr (DK) *dk = false;
   T off_last = T(0);
   int sweep = 0;
@@ -706,29 +758,11 @@ __device__ int jacobi_herm(T* Ar, T* Ai, T* Vr, T* Vi, T* cs, T* red, int tid, b
       }
     }
     for (int r = 0; r < n - 1; ++r) {
-      // the rotation of each pair, and the pair's own 2x2 block made (real) diagonal
-      for (int k = tid; k < H; k += NT) {
-        int p, q;
-        rr_pair(n, r, k, p, q);
-        const T app = Ar[p * LD + p], aqq = Ar[q * LD + q];
-        const T br = Ar[p * LD + q], bi = Ai[p * LD + q];
-        T c, s, t, mag = T(0), wr = T(1), wi = T(0);
-        if (br != T(0) || bi != T(0)) unit_phase<T>(br, bi, mag, wr, wi);
-        sym_schur2<T>(app, aqq, mag, c, s, t);
-        cs[k] = c;
-        cs[H + k] = s;
-        cs[2 * H + k] = wr;
-        cs[3 * H + k] = wi;
-        Ar[p * LD + p] = app - t * mag;
-        Ar[q * LD + q] = aqq + t * mag;
-        Ai[p * LD + p] = T(0);
-        Ai[q * LD + q] = T(0);
-        Ar[p * LD + q] = T(0);
-        Ai[p * LD + q] = T(0);
-        Ar[q * LD + p] = T(0);
-        Ai[q * LD + p] = T(0);
+      cs = (r & 1) ? cs2 : cs1;
+      if (!PIPE || r == 0) {
+        rotations(r, cs);
+        gsync<NT>();
       }
-      gsync<NT>();
       if constexpr (!ROWS) {
       // the blocks (k1, k2), k1 < k2 (pairs of a circle ordering of the H pair indices), and
       // their conjugate transposes (k2, k1)
@@ -860,13 +894,18 @@ __device__ int jacobi_herm(T* Ar, T* Ai, T* Vr, T* Vi, T* cs, T* red, int tid, b
           }
         }
       }
+      if constexpr (PIPE) {
+        gsync<NT>();
+        if (r + 1 < n - 1) rotations(r + 1, (r & 1) ? cs1 : cs2);
+      }
       if constexpr (VEC) {
-        for (int t0 = tid; t0 < n * H; t0 += GV * NT) {
+        constexpr int VT = PIPE ? NT - 32 : NT;
+        for (int t0 = !PIPE ? tid : tid < 32 ? n * H : tid - 32; t0 < n * H; t0 += GV * VT) {
           int ix[GV], kk[GV], pp[GV], qq[GV];
           T vpr[GV], vpi[GV], vqr[GV], vqi[GV];
 #pragma unroll
           for (int g = 0; g < GV; ++g) {
-            const int t = t0 + g * NT;
+            const int t = t0 + g * VT;
             if (t < n * H) {
               ix[g] = LANE_ROWS ? t % n : t / H;
               kk[g] = LANE_ROWS ? t / n : t % H;
@@ -879,7 +918,7 @@ __device__ int jacobi_herm(T* Ar, T* Ai, T* Vr, T* Vi, T* cs, T* red, int tid, b
           }
 #pragma unroll
           for (int g = 0; g < GV; ++g) {
-            if (t0 + g * NT >= n * H) continue;
+            if (t0 + g * VT >= n * H) continue;
             const int k = kk[g];
             const T c = cs[k], s = cs[H + k], wr = cs[2 * H + k], wi = cs[3 * H + k];
             // v_p' = c v_p - s w v_q ; v_q' = s v_p + c w v_q
