@@ -477,7 +477,7 @@ __device__ int jacobi_sym(T* A, T* V, T* cs, T* red, int tid, bool* dk = nullptr
     }
   }
   // the rotations of round r + 1 by the first warp while the others update V for round r: they are a
-  // serial chain of divides and square roots on H lanes (64 x 64 float32, 25 matrices: 258 -> 243 us
+  // serial chain of divides and square roots on H lanes (64 x 64 float32, 25 clusters: 258 -> 243 us
   // real, 384 -> 357 us complex)
   constexpr bool PIPE = VEC && LANE_ROWS && NT > 32;
   T* cs2 = cs;
