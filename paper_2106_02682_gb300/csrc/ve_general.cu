@@ -1157,8 +1157,11 @@ int ve_general_bound(ve_general* h, ve_cert* out) {
   VG_CU(launch_gbound_pair(a, h->lmin_p, s));
   VG_CU(launch_small(a, 2, h->lmin_c, s));
   // lmin(X): the eigensolve starts from the last bound's eigenvectors
-  VG_CU(dense_eig(h->bws, h->X, h->bounds % kRefresh ? DENSE_WARM : DENSE_COLD, s));
-  ++h->bounds;
+  // (from V = I again after one that did not end in a finite bound: its eigenvectors may not be)
+  const int mode = h->bounds % kRefresh ? DENSE_WARM : DENSE_COLD;
+  const long next = h->bounds + 1;
+  h->bounds = 0;
+  VG_CU(dense_eig(h->bws, h->X, mode, s));
   VG_CU(dense_lmin_certified(h->bws, s));
   std::vector<double> lp((size_t)h->K), lc((size_t)h->N);
   DenseCtl ctl;
@@ -1174,6 +1177,7 @@ int ve_general_bound(ve_general* h, ve_cert* out) {
   const double xmin = ctl.lmin;
   // every minimum passes a NaN on, and an Inf stays in the sum: one check covers them all
   if (!std::isfinite(raw) || !std::isfinite(xmin)) return VE_ENONFINITE;
+  h->bounds = next;
   const double corr = (double)h->N * h->m * (xmin < 0 ? -xmin : 0.0);
   out->raw_bound = raw;
   out->x_min_eig = xmin;

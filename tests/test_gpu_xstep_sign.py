@@ -55,3 +55,26 @@ def test_one_sweep_matches_the_oracle(spins, L, kind):
     assert np.max(np.abs(got - st['X'])) <= 1e-10 * max(1.0, n / 64) * scale
     assert np.array_equal(got, got.T)
     assert np.array_equal(again[-n * n:].reshape(n, n), got)
+
+
+def test_bound_after_a_bound_of_a_nonfinite_state():
+    """The bound's eigensolve of X starts from the last bound's eigenvectors, but not from those of a
+    state that was not finite."""
+    from paper_2106_02682_gb300 import ve
+    terms = synth.disordered_chain(6, "tfim", seed=3)
+    h = ve.ve_general_create(terms, 1, ve.ve_default_options())
+    try:
+        ve.ve_general_iterate(h, 5)
+        good = ve.ve_general_get_state(h)
+        want = ve.ve_general_bound(h).bound_per_spin
+        bad = good.copy()
+        bad[-1] = np.nan  # an entry of X
+        ve.ve_general_set_state(h, bad)
+        with pytest.raises(ve.VEError):
+            ve.ve_general_bound(h)
+        ve.ve_general_set_state(h, good)
+        got = ve.ve_general_bound(h)
+    finally:
+        ve.ve_general_destroy(h)
+    # the pair and cluster minima do not depend on X; its own enters with N m max(0, -lmin(X))
+    assert abs(got.bound_per_spin - want) <= 1e-11
