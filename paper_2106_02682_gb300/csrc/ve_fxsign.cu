@@ -74,6 +74,15 @@ __device__ __forceinline__ void write_block(const Frag& z, uint4* out, int nb, i
   }
 }
 
+// Each kernel of the chain lets the next one's CTAs start beside it (they wait here until it has
+// finished and its writes are visible, before their first access to global memory).  Every kernel
+// waits here, so whatever is two launches back has finished as well.  Measured a sweep, without / with:
+// n = 512 810 / 783 us, n = 160 252 / 248 us.
+__device__ __forceinline__ void after_previous() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // One product.  A CTA holds TB x TB output blocks of 16 x 16 (blocks TB bi .., TB bj .., bi <= bj),
 // KW warps a block sharing its K range.
 template <int MODE, int TB>
@@ -87,6 +96,7 @@ __global__ void __launch_bounds__(32 * kWarps, 1) k_fx_product(const Args p) {
   int bi, bj;
   tri_index(T, blockIdx.x, bi, bj);
   const int I = bi * TB + blk / TB, J = bj * TB + blk % TB;
+  after_previous();
   const bool live = I <= J && J < p.nb;
   Frag h = {};
   if (live) {
@@ -226,6 +236,7 @@ __global__ void __launch_bounds__(256) k_fx_norm(const double* __restrict__ Y, i
 __global__ void __launch_bounds__(256) k_fx_slice(const double* __restrict__ Y, int n, int nb, const double* partial,
                                                   uint4* X, uint4* Yq, FxSignCtl* ctl, int* ey) {
   const int lane = threadIdx.x & 31;
+  after_previous();
   double v = 0.0, m = 0.0;
   for (int k = lane; k < kNormCtas; k += 32) {
     v += partial[k];
@@ -264,6 +275,7 @@ __global__ void __launch_bounds__(256) k_fx_slice(const double* __restrict__ Y, 
 // The convergence test: block residuals added in a fixed order.
 __global__ void __launch_bounds__(256) k_fx_check(const double* partial, int nb, FxSignCtl* ctl) {
   __shared__ double red[8];
+  after_previous();
   double v = 0.0;
   for (int e = threadIdx.x; e < nb * nb; e += 256)
     if (e / nb <= e % nb) v += partial[e];
@@ -274,17 +286,28 @@ __global__ void __launch_bounds__(256) k_fx_check(const double* partial, int nb,
   }
 }
 
+// A launch that need not wait for the one before it on the stream to finish (after_previous).
+template <class... P, class... A>
+cudaError_t launch_after(void (*f)(P...), int grid, int threads, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3((unsigned)grid);
+  c.blockDim = dim3((unsigned)threads);
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, f, P(args)...);
+}
+
 // 32 x 32 tiles where they fill the chip; else one block a CTA with its K range shared by all the
 // warps (n = 160: 55 CTAs instead of 15).
 template <int MODE>
 cudaError_t launch(const Args& a, cudaStream_t s) {
   const int T = (a.nb + 1) / 2;
-  if (T * (T + 1) / 2 >= 100) {
-    k_fx_product<MODE, 2><<<T * (T + 1) / 2, 32 * kWarps, 0, s>>>(a);
-  } else {
-    k_fx_product<MODE, 1><<<a.nb * (a.nb + 1) / 2, 32 * kWarps, 0, s>>>(a);
-  }
-  return cudaGetLastError();
+  if (T * (T + 1) / 2 >= 100) return launch_after(k_fx_product<MODE, 2>, T * (T + 1) / 2, 32 * kWarps, s, a);
+  return launch_after(k_fx_product<MODE, 1>, a.nb * (a.nb + 1) / 2, 32 * kWarps, s, a);
 }
 
 size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -321,8 +344,7 @@ cudaError_t issue_pass(FxSignWs& w, const double* Y, double* X, cudaStream_t s) 
   a.A = w.X[0];
   a.B = w.Yq;
   if ((e = launch<kFinal>(a, s)) != cudaSuccess) return e;
-  k_fx_check<<<1, 256, 0, s>>>(a.partial, w.nb, w.ctl);
-  return cudaGetLastError();
+  return launch_after(k_fx_check, 1, 256, s, a.partial, w.nb, w.ctl);
 }
 
 cudaError_t build_graph(FxSignWs& w, const double* Y, double* X, bool first, cudaGraphExec_t* out) {
@@ -334,9 +356,10 @@ cudaError_t build_graph(FxSignWs& w, const double* Y, double* X, bool first, cud
     if (first) {
       k_fx_norm<<<kNormCtas, 256, 0, cs>>>(Y, w.n, w.partial);
       const int blocks = w.nb * (w.nb + 1) / 2;
-      k_fx_slice<<<(blocks + 7) / 8, 256, 0, cs>>>(Y, w.n, w.nb, w.partial, w.X[0], w.Yq, w.ctl,
-                                                   reinterpret_cast<int*>(w.ctl + 1));
       e = cudaGetLastError();
+      if (e == cudaSuccess)
+        e = launch_after(k_fx_slice, (blocks + 7) / 8, 256, cs, Y, w.n, w.nb, w.partial, w.X[0], w.Yq, w.ctl,
+                         reinterpret_cast<int*>(w.ctl + 1));
     }
     if (e == cudaSuccess) e = issue_pass(w, Y, X, cs);
     cudaGraph_t g = nullptr;
