@@ -90,7 +90,7 @@ __device__ __forceinline__ long long fix(double v, int E) {
   m = shift_round(m, E - (e ? e : 1));
   return b < 0 ? -m : m;
 }
-// x 2^e, |x| < 2^62, rounded to nearest; results below the normal range become 0.
+// x 2^e, |x| < 2^62, rounded to nearest (halves away from zero).
 __device__ __forceinline__ double word(long long x, int e) {
   unsigned long long a = (unsigned long long)(x < 0 ? -x : x);
   if (a == 0) return 0.0;
@@ -107,7 +107,10 @@ __device__ __forceinline__ double word(long long x, int e) {
   }
   const int sh = lz - 11, ex = e - sh + 1075;
   const unsigned long long sign = x < 0 ? 1ULL << 63 : 0;
-  if (ex <= 0) return 0.0;
+  if (ex <= 0) {  // subnormal
+    if (ex < -52) return 0.0;
+    return __longlong_as_double((long long)(sign | (((a << sh) + (1ULL << -ex)) >> (1 - ex))));
+  }
   if (ex >= 0x7ff) return __longlong_as_double((long long)(sign | (0x7ffULL << 52)));
   return __longlong_as_double((long long)(sign | ((unsigned long long)ex << 52) | ((a << sh) & 0xfffffffffffffULL)));
 }
@@ -834,7 +837,7 @@ __device__ double lowest(Frag& ar, Frag& ai, int ea, unsigned char* sm, int lane
   for (int o = 16; o > 0; o >>= 1) w = nan_min(w, shfl_xor(w, o));
   __syncwarp();
   // the sum was taken in float32: rounded up by more than its error
-  return w - 9007199254740992.0 * (double)(sqrtf(off2) * 1.0001f) * word(1, ea);
+  return w - 2.0 * (double)(sqrtf(off2) * 1.0001f) * word(1LL << 52, ea);
 }
 
 }  // namespace fx16
