@@ -118,30 +118,33 @@ __device__ __forceinline__ void product(const uint4* A, const uint4* B, int I, i
   }
 }
 
-// Sum and largest value over the CTA.
-__device__ __forceinline__ void reduce(double& v, int& m, unsigned char* red, int tid) {
+// Sum, and largest value, over the CTA.
+__device__ __forceinline__ double reduce_sum(double v, unsigned char* red, int tid) {
   double* rv = reinterpret_cast<double*>(red);
-  int* rm = reinterpret_cast<int*>(red + kWarps * 8);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += shfl_xor(v, o);
-  m = (int)__reduce_max_sync(0xffffffffu, (unsigned)m);
   __syncthreads();
-  if ((tid & 31) == 0) {
-    rv[tid >> 5] = v;
-    rm[tid >> 5] = m;
-  }
+  if ((tid & 31) == 0) rv[tid >> 5] = v;
   __syncthreads();
   v = 0.0;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) v += rv[w];
+  return v;
+}
+__device__ __forceinline__ int reduce_max(int m, unsigned char* red, int tid) {
+  int* rm = reinterpret_cast<int*>(red + kWarps * 8);
+  m = (int)__reduce_max_sync(0xffffffffu, (unsigned)m);
+  __syncthreads();
+  if ((tid & 31) == 0) rm[tid >> 5] = m;
+  __syncthreads();
   m = 0;
 #pragma unroll
-  for (int w = 0; w < kWarps; ++w) {
-    v += rv[w];
-    m = max(m, rm[w]);
-  }
+  for (int w = 0; w < kWarps; ++w) m = max(m, rm[w]);
+  return m;
 }
 
 // load(row, col, re, im): entry of the matrix C, Hermitian when taken on and above the diagonal
-// (called twice an entry); store(row, col, re, im): entry of the result, all of them (after a
+// (called five times an entry); store(row, col, re, im): entry of the result, all of them (after a
 // barrier: it may overwrite what load reads and the first Smem::matrix bytes of sm).  All threads
 // call; ends with a barrier.  Returns the passes; a non-finite C gives NaN throughout.
 template <bool CPLX, class Load, class Store>
@@ -166,18 +169,28 @@ __device__ int project(unsigned char* sm, int tid, Load load, Store store) {
     }
   };
   Frag hr, hi;
-  double nrm = 0.0;
+  // ||C||_F of the entries scaled by the largest one's binade: squares that neither overflow nor vanish
   int E = 0;
 #pragma unroll 1
   for (int i = 0; i < 8; ++i) {
     double re, im;
     entry(i, re, im);
-    nrm += (I == J ? 1.0 : 2.0) * fma(re, re, CPLX ? im * im : 0.0);
     E = max(E, fx16::exponent_field(re));
     if constexpr (CPLX) E = max(E, fx16::exponent_field(im));
   }
-  reduce(nrm, E, red, tid);
-  const bool finite = E != 0x7ff && isfinite(nrm);
+  E = reduce_max(E, red, tid);
+  const bool finite = E != 0x7ff;
+  const double unit = fxstep::binade_scale(E);
+  double nrm = 0.0;
+#pragma unroll 1
+  for (int i = 0; i < 8; ++i) {
+    double re, im;
+    entry(i, re, im);
+    re *= unit;
+    im *= unit;
+    nrm += (I == J ? 1.0 : 2.0) * fma(re, re, CPLX ? im * im : 0.0);
+  }
+  nrm = reduce_sum(nrm, red, tid);
   int pass = 0;
   if (finite && nrm > 0.0) {
     const double inv = (1.0 - 1e-9) * 9007199254740992.0 / sqrt(nrm);
@@ -185,8 +198,8 @@ __device__ int project(unsigned char* sm, int tid, Load load, Store store) {
     for (int i = 0; i < 8; ++i) {
       double re, im;
       entry(i, re, im);
-      hr[i] = __double2ll_rn(re * inv);
-      if constexpr (CPLX) hi[i] = __double2ll_rn(im * inv);
+      hr[i] = __double2ll_rn(re * unit * inv);
+      if constexpr (CPLX) hi[i] = __double2ll_rn(im * unit * inv);
     }
     write_block<CPLX>(hr, hi, X, I, J, lane);
     __syncthreads();
@@ -212,10 +225,7 @@ __device__ int project(unsigned char* sm, int tid, Load load, Store store) {
         write_block<CPLX>(yr, yi, Z, I, J, lane);
         __syncthreads();
         if (k == fxstep::kSteps - 1) {
-          double v = (I == J ? 1.0 : 2.0) * (double)res;
-          int none = 0;
-          reduce(v, none, red, tid);
-          done = v <= fxstep::kResid;
+          done = reduce_sum((I == J ? 1.0 : 2.0) * (double)res, red, tid) <= fxstep::kResid;
         }
         // a I + b X^2 + c X^4, units of 2^-50
         product<CPLX>(Z, Z, I, J, hr, hi, lane);

@@ -52,6 +52,12 @@ constexpr Coef coef(int k) {
 // x c for |c| < 64 given in units of 2^-56, |x| < 2^55.
 __device__ __forceinline__ long long scale(long long x, long long c) { return __mul64hi(x << 8, c); }
 
+// The power of two that brings a number of exponent field E into [1, 4); a subnormal one (E = 0) to
+// 2^-51 at least.  A product with it is exact.
+__device__ __forceinline__ double binade_scale(int E) {
+  return __hiloint2double((E < 2045 ? 2046 - E : 1) << 20, 0);
+}
+
 __device__ __forceinline__ uint32_t transpose8(uint32_t v) {
   uint32_t r;
   asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(v));

@@ -50,3 +50,8 @@ def _check_x_step(D, exponent):
 @pytest.mark.parametrize("exponent", SCALES)
 def test_x_step_16(exponent):
     _check_x_step(16, exponent)
+
+
+@pytest.mark.parametrize("exponent", SCALES)
+def test_x_step_64(exponent):
+    _check_x_step(64, exponent)
