@@ -214,7 +214,8 @@ __global__ void __launch_bounds__(32 * kWarps, 1) k_fx_product(const Args p) {
   }
 }
 
-// Per-CTA sums of squares and largest entries of Y.
+// Per-CTA largest entries of Y, and sums of squares of the entries scaled by the CTA's largest one's
+// binade: in one pass (the power of two applied to the sum) where the squares stay in range, else in two.
 __global__ void __launch_bounds__(256) k_fx_norm(const double* __restrict__ Y, int n, double* partial) {
   __shared__ double red[8];
   const size_t nn = (size_t)n * n;
@@ -223,8 +224,17 @@ __global__ void __launch_bounds__(256) k_fx_norm(const double* __restrict__ Y, i
     v = fma(Y[e], Y[e], v);
     m = fmax(m, fabs(Y[e]));
   }
-  v = gsum<256>(v, red);
   m = -gmin<256>(-m, red);
+  const int E = fx16::exponent_field(m);
+  const double unit = binade_scale(E);
+  if (E > 623 && E < 1423) {
+    v = v * unit * unit;
+  } else {
+    v = 0.0;
+    for (size_t e = blockIdx.x * (size_t)256 + threadIdx.x; e < nn; e += (size_t)gridDim.x * 256)
+      v = fma(Y[e] * unit, Y[e] * unit, v);
+  }
+  v = gsum<256>(v, red);
   if (threadIdx.x == 0) {
     partial[blockIdx.x] = v;
     partial[kNormCtas + blockIdx.x] = m;
@@ -238,17 +248,19 @@ __global__ void __launch_bounds__(256) k_fx_slice(const double* __restrict__ Y, 
   const int lane = threadIdx.x & 31;
   after_previous();
   double v = 0.0, m = 0.0;
-  for (int k = lane; k < kNormCtas; k += 32) {
-    v += partial[k];
-    m = fmax(m, partial[kNormCtas + k]);
+  for (int k = lane; k < kNormCtas; k += 32) m = fmax(m, partial[kNormCtas + k]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, shfl_xor(m, o));
+  const int E = fx16::exponent_field(m);  // Yq: an entry of the largest one's binade is 2^52 .. 2^53
+  for (int k = lane; k < kNormCtas; k += 32) {  // from the CTA's scale to the matrix's
+    const int d = binade_field(E) - binade_field(fx16::exponent_field(partial[kNormCtas + k]));  // <= 0
+    const double c = d > -1023 ? __hiloint2double((1023 + d) << 20, 0) : 0.0;
+    v += partial[k] * c * c;
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    v += shfl_xor(v, o);
-    m = fmax(m, shfl_xor(m, o));
-  }
+  for (int o = 16; o > 0; o >>= 1) v += shfl_xor(v, o);
   const bool finite = isfinite(v) != 0;
-  const int E = fx16::exponent_field(m);  // Yq: an entry of the largest one's binade is 2^52 .. 2^53
+  const double unit = binade_scale(E);
   const double inv = finite && v > 0.0 ? (1.0 - 1e-9) * 9007199254740992.0 / sqrt(v) : 0.0;
   const long w = (long)blockIdx.x * 8 + (threadIdx.x >> 5);
   if (w == 0 && lane == 0) {
@@ -265,7 +277,7 @@ __global__ void __launch_bounds__(256) k_fx_slice(const double* __restrict__ Y, 
     const int row = 16 * I + fx16::frag_row(i, lane), col = 16 * J + fx16::frag_col(i, lane);
     double y = 0.0;
     if (finite && row < n && col < n) y = 0.5 * (Y[(size_t)row * n + col] + Y[(size_t)col * n + row]);
-    x[i] = __double2ll_rn(y * inv);
+    x[i] = __double2ll_rn(y * unit * inv);
     q[i] = fx16::fix(y, E);
   }
   write_block(x, X, nb, I, J, lane);

@@ -9,7 +9,7 @@
 namespace ve {
 
 struct FxSignCtl {
-  double fro2;     // ||Y||_F^2
+  double fro2;     // ||Y||_F^2, Y scaled by its largest entry's binade
   double resid;    // ||I - X^2||_F^2 before the last step
   int done;        // the sign has converged (or Y is zero or not finite)
   int finite;

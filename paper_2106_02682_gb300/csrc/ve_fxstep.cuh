@@ -54,9 +54,8 @@ __device__ __forceinline__ long long scale(long long x, long long c) { return __
 
 // The power of two that brings a number of exponent field E into [1, 4); a subnormal one (E = 0) to
 // 2^-51 at least.  A product with it is exact.
-__device__ __forceinline__ double binade_scale(int E) {
-  return __hiloint2double((E < 2045 ? 2046 - E : 1) << 20, 0);
-}
+__device__ __forceinline__ int binade_field(int E) { return E < 2045 ? 2046 - E : 1; }
+__device__ __forceinline__ double binade_scale(int E) { return __hiloint2double(binade_field(E) << 20, 0); }
 
 __device__ __forceinline__ uint32_t transpose8(uint32_t v) {
   uint32_t r;

@@ -55,3 +55,28 @@ def test_x_step_16(exponent):
 @pytest.mark.parametrize("exponent", SCALES)
 def test_x_step_64(exponent):
     _check_x_step(64, exponent)
+
+
+@pytest.mark.parametrize("exponent", [-1018, -560, 530])
+@pytest.mark.parametrize("spins", [5, 26])
+def test_dense_x_step(spins, exponent):
+    """One sweep of the general solver, its global step so weak that Y = X to rounding."""
+    from paper_2106_02682_gb300 import synth, ve
+    n = 4 * spins
+    rng = np.random.default_rng(spins)
+    Q, _ = np.linalg.qr(rng.normal(size=(n, n)))
+    X = (Q * rng.uniform(-1.0, 1.0, n)) @ Q.T
+    X = 0.5 * (X + X.T)
+    h = ve.ve_general_create(synth.disordered_chain(spins, "xxz", seed=spins), 1, ve.ve_default_options(eps=1e-323))
+    try:
+        state = ve.ve_general_get_state(h)
+        state[-n * n:] = np.ldexp(X, exponent).ravel()
+        ve.ve_general_set_state(h, state)
+        try:
+            ve.ve_general_iterate(h, 1)
+        except ve.VEError:
+            assert exponent > 500  # the feasibility error is a sum of squares
+        got = np.ldexp(ve.ve_general_get_state(h)[-n * n:].reshape(n, n), -exponent)
+    finally:
+        ve.ve_general_destroy(h)
+    assert np.max(np.abs(got - _psd(X))) <= 64 * n * U
