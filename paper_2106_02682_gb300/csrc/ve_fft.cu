@@ -680,6 +680,33 @@ __global__ void __launch_bounds__(32, 16)
       atomicAdd(stats + 1, 1ull);
       if (dk) atomicAdd(stats + 2, 1ull);
     }
+    // A definite block comes back as the Hermitian part of C_k itself, like the others: rounding that
+    // breaks X_{-delta} = X_delta^T would add up over the sweeps otherwise.  In rolled loops, through
+    // shared memory: the path is rare.
+    if (finite && res == fx16::kSame) {
+      double2* buf = reinterpret_cast<double2*>(smem_raw);
+      __syncwarp();
+#pragma unroll 1
+      for (int e = lane; e < E; e += 32) {
+        double hr[2], hi[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {  // entry (r + 8 h, c) and its transpose
+          const int r = (e >> 4) + 8 * h, c = e & 15, t = (c & 7) * 16 + r;
+          const double2 z = z1[e], zz = z2[e], w = z1[t], ww = z2[t];
+          hr[h] = 0.25 * ((h ? z.y + zz.y : z.x + zz.x) + (c < 8 ? w.x + ww.x : w.y + ww.y));
+          hi[h] = 0.25 * ((h ? zz.x - z.x : z.y - zz.y) - (c < 8 ? w.y - ww.y : ww.x - w.x));
+        }
+        buf[e] = make_double2(hr[0] - hi[1], hi[0] + hr[1]);
+        buf[E + e] = make_double2(hr[0] + hi[1], hr[1] - hi[0]);
+      }
+      __syncwarp();
+#pragma unroll 1
+      for (int e = lane; e < E; e += 32) {
+        z1[e] = buf[e];
+        if (s2 != s) z2[e] = buf[E + e];
+      }
+      __syncwarp();
+    }
     // pack Y_k (and Y_{-k} = conj Y_k) back, scaled by 1/N
     const double sc = finite ? (res == fx16::kProduct && pow2 ? 1.0 : res == fx16::kZero ? 0.0 : invN) : NAN;
     if (pow2) ea -= log2n;
@@ -691,7 +718,7 @@ __global__ void __launch_bounds__(32, 16)
       if (finite && res == fx16::kProduct) {
         a = make_double2(fx16::word(ar[k] - ai[k + 2], ea), fx16::word(ai[k] + ar[k + 2], ea));
         b = make_double2(fx16::word(ar[k] + ai[k + 2], ea), fx16::word(ar[k + 2] - ai[k], ea));
-      } else {  // C_k itself (definite), zero, or NaN throughout
+      } else {  // definite, zero, or NaN throughout
         a = z1[e];
         b = z2[e];
       }
