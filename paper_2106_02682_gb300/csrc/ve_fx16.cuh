@@ -49,7 +49,7 @@ using Frag = long long[8];  // one real 16 x 16 matrix, A-fragment layout
 template <bool CPLX>
 struct Smem {
   static constexpr size_t region = (CPLX ? 2 : 1) * (size_t)kD * 512;
-  static constexpr size_t lam = 2 * region;  // 16 float32 eigenvalues; (EIG) 16 low parts of them
+  static constexpr size_t lam = 2 * region;  // 16 eigenvalues as float32 pairs: high parts, low parts
   static constexpr size_t bytes = lam + 128;
   static constexpr size_t vectors = (CPLX ? 2 : 1) * 256 * 8;  // an eigenvector store of 8-byte words
   static_assert((CPLX ? 2 : 1) * 16 * kLd * 8 <= region && (CPLX ? 4 : 2) * 16 * kLd * 4 <= region, "regions");
@@ -639,6 +639,23 @@ __device__ void update_vectors(long long* v, const float* Qr, const float* Qi, u
   }
 }
 
+// x times the divided difference of max(., 0) between p = ph + pl >= 0 and -q, q = qh + ql > 0, which is
+// w = p / (p + q).  x is at most 6e-8 of the matrix where the first-order rule has just been met, so w to
+// 2^-31 leaves less than a rounding of x; float32 alone (1e-7) left up to 5 u ||A|| there.
+__device__ __forceinline__ int cross_weight(float ph, float pl, float qh, float ql) {  // units of 2^-30
+  float dh, dl;
+  two_sum(ph, qh, dh, dl);
+  dl += pl + ql;
+  const float inv = __fdividef(1.f, dh), w = ph * inv;
+  const float r = fmaf(-w, dh, ph) + fmaf(-w, dl, pl);
+  return __float2int_rn(w * 1073741824.f) + __float2int_rn(r * inv * 1073741824.f);
+}
+__device__ __forceinline__ long long weighted(long long x, int w) {
+  const long long hi = (long long)(int)(x >> 32) * w;
+  const unsigned long long lo = (unsigned long long)(uint32_t)x * (uint32_t)w;
+  return (hi << 2) + (long long)((lo + (1ULL << 29)) >> 30);
+}
+
 // Y is in the fragments; Y = C; Y = 0; (EIG) A = V^H C V is in the fragments
 enum Result { kProduct, kSame, kZero, kDiagonal };
 
@@ -764,7 +781,11 @@ __device__ Result project(Frag& ar, Frag& ai, int& ea, long long* v, bool warm, 
       if (neg == 0u || neg == 0xffffffffu) return neg ? kZero : kSame;
     }
     if (!EIG && (*dk || f.off <= 3.1554436e-30f * f.nrm2() /* (n u)^2 */ || cyc == kMaxCycles)) {
-      // M = f(Lambda) + L o E (dk_weight), conjugated, into region 1
+      // M = f(Lambda) + L o E, conjugated, into region 1
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (frag_row(k, lane) == frag_col(k, lane)) lam[16 + frag_row(k, lane)] = unit_float(ar[k] - unit_fix(xf[k]));
+      __syncwarp();
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
         const int i = frag_row(k, lane), j = frag_col(k, lane);
@@ -773,9 +794,11 @@ __device__ Result project(Frag& ar, Frag& ai, int& ea, long long* v, bool warm, 
           ar[k] = ar[k] > 0 ? ar[k] : 0;
           if constexpr (CPLX) ai[k] = 0;
         } else if (li < 0.f || lj < 0.f) {
-          const float w = li >= 0.f || lj >= 0.f ? fmaxf(li, lj) / (fabsf(li) + fabsf(lj)) : 0.f;
-          ar[k] = unit_fix(xf[k] * w);
-          if constexpr (CPLX) ai[k] = unit_fix(yf[k] * w);
+          const bool up = li >= lj;
+          const float pl = lam[16 + (up ? i : j)], ql = -lam[16 + (up ? j : i)];
+          const int w = (li < 0.f) != (lj < 0.f) ? cross_weight(fmaxf(li, lj), pl, -fminf(li, lj), ql) : 0;
+          ar[k] = weighted(ar[k], w);
+          if constexpr (CPLX) ai[k] = weighted(ai[k], w);
         }
         if constexpr (CPLX) ai[k] = -ai[k];
       }
