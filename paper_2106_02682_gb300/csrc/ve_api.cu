@@ -272,8 +272,11 @@ SmallArgs small_args(ve_handle* h) {
   return a;
 }
 
-// One sweep of Algorithm 6, all on h->stream (with stage events when profiling).
-cudaError_t issue_sweep(ve_handle* h, int arith, bool warm) {
+constexpr int kBranchBatch = 8;
+
+// One sweep of Algorithm 6, on h->stream (with stage events when profiling) and, where `branch` allows it,
+// a branch beside it.
+cudaError_t issue_sweep(ve_handle* h, int arith, bool warm, bool branch = true) {
   cudaStream_t s = h->stream;
   const int v = arith;
   const bool fp32 = arith == ARITH_FP32;
@@ -302,8 +305,11 @@ cudaError_t issue_sweep(ve_handle* h, int arith, bool warm) {
   // Lambda1, Lambda2 and the status need rho_0 only, and nothing before the next sweep needs them.
   // Small instances leave SMs idle and run them on a branch beside the X step; large ones in line,
   // where the branch costs more than its 10 us (measured, us a sweep, branch / line: 16 clusters 60
-  // / 66, 50 clusters 153 / 159, 2048 clusters 253 / 230, 4096 clusters 372 / 345).
-  const bool beside = !h->prof && h->Pc <= 2 * big_grid();
+  // / 66, 50 clusters 153 / 159, 2048 clusters 253 / 230, 4096 clusters 372 / 345).  In a batch the
+  // instances run beside each other anyway, and past kBranchBatch of them a second branch an instance
+  // costs more in the graph than it hides (2-spin clusters, mixed, us a sweep of the batch, branch / line:
+  // 4 instances 71 / 79, 8 instances 88 / 92, 16 instances 145 / 123, 24 instances 247 / 164).
+  const bool beside = branch && !h->prof && h->Pc <= 2 * big_grid();
   const cudaStream_t q = beside ? h->side : s;
   if (beside) {
     if ((e = cudaEventRecord(h->fork, s)) != cudaSuccess) return e;
@@ -1063,7 +1069,7 @@ void batch_drop_graph(ve_batch* b) {
 
 // One graph whose branches are one sweep of every instance with key >= 0 (fork on the main
 // stream, one branch per instance stream, join back).
-int batch_capture(ve_batch* b, const std::vector<int>& key) {
+int batch_capture(ve_batch* b, const std::vector<int>& key, bool branch) {
   batch_drop_graph(b);
   VE_CU(cudaStreamBeginCapture(b->main, cudaStreamCaptureModeThreadLocal));
   cudaError_t e = cudaEventRecord(b->fork, b->main);
@@ -1071,7 +1077,7 @@ int batch_capture(ve_batch* b, const std::vector<int>& key) {
     if (key[i] < 0) continue;
     ve_handle* h = b->h[i];
     e = cudaStreamWaitEvent(h->stream, b->fork, 0);
-    if (e == cudaSuccess) e = issue_sweep(h, key[i], true);
+    if (e == cudaSuccess) e = issue_sweep(h, key[i], true, branch);
     if (e == cudaSuccess) e = cudaEventRecord(b->join[i], h->stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(b->main, b->join[i], 0);
   }
@@ -1154,16 +1160,18 @@ int ve_batch_iterate(ve_batch* b, long max_iter, double tol, ve_status* out) {
   while (done < max_iter) {
     const long chunk = (long)check < max_iter - done ? (long)check : max_iter - done;
     std::vector<int> key(n, -1);
-    bool any = false, cold = false;
+    int active = 0;
+    bool cold = false;
     for (int i = 0; i < n; ++i) {
       if (ctl[i].finished) continue;
       ve_handle* h = b->h[i];
       if (h->prof) return VE_EINVAL;  // per-stage profiling is per handle, not in a batch
       key[i] = handle_arith(h);
-      any = true;
+      ++active;
       if (!h->vvalid[key[i]]) cold = true;
     }
-    if (!any) break;
+    if (!active) break;
+    const bool branch = active <= kBranchBatch;
     long launches = chunk;
     if (cold) {
       // some instance starts a precision phase: its first sweep runs directly and cold (as in
@@ -1173,7 +1181,7 @@ int ve_batch_iterate(ve_batch* b, long max_iter, double tol, ve_status* out) {
         if (key[i] < 0) continue;
         ve_handle* h = b->h[i];
         const int v = key[i];
-        VE_CU(issue_sweep(h, v, h->vvalid[v]));
+        VE_CU(issue_sweep(h, v, h->vvalid[v], branch));
         h->vvalid[v] = true;
         VE_CU(cudaEventRecord(b->join[i], h->stream));
         VE_CU(cudaStreamWaitEvent(b->main, b->join[i], 0));
@@ -1181,7 +1189,7 @@ int ve_batch_iterate(ve_batch* b, long max_iter, double tol, ve_status* out) {
       --launches;
     }
     if (launches > 0 && (!b->exec || key != b->key)) {
-      const int r = batch_capture(b, key);
+      const int r = batch_capture(b, key, branch);
       if (r != VE_OK) return r;
     }
     for (long c = 0; c < launches; ++c) VE_CU(cudaGraphLaunch(b->exec, b->main));
