@@ -335,8 +335,8 @@ int ve_selftest_bounded_wait(double* seconds);
  * No translation invariance: random fields, inhomogeneous or long-range couplings.  Every
  * cluster i has its own H_i and rho_i, every pair i < j its own H_ij, rho~_ij, Lambda_ij,
  * Lambda1_ij, Lambda2_ij, and X is one dense (N D) x (N D) matrix whose projection X <-
- * Pi_{>=0}(X - eps G) runs over the whole GPU as (Y + sign(Y) Y) / 2, Y = X - eps G, the matrix
- * sign by a polynomial iteration of float64-accurate products on the tensor cores.
+ * Pi_{>=0}(X - eps G) runs over the whole GPU as P Y P, Y = X - eps G, P = (I + sign(Y)) / 2, the
+ * matrix sign by a polynomial iteration of float64-accurate products on the tensor cores.
  * The X step takes the ascent sign X - eps G, as ve_create's solver does.
  *
  * The Hamiltonian is a list of terms on nspins spins:
@@ -434,8 +434,8 @@ int ve_general_set_state(ve_general* h, const double* host, size_t bytes);
 #define VE_GENERAL_NSTAGE 4
 int ve_general_profile(ve_general* h, int enable);
 int ve_general_profile_read(ve_general* h, double* ms, long* launches, double* jacobi_sweeps);
-/* Device time of the profiled X steps and the launches they held (36 products a pass, two launches
- * before and two after them); *first_order is 0. */
+/* Device time of the profiled X steps and the launches they held (38 products a pass, four launches
+ * beside them); *first_order is 0. */
 int ve_general_profile_rounds(ve_general* h, double* ms, long* rounds, long* first_order);
 
 /* Pi_{>=0} of ONE real symmetric n x n matrix (device, row-major; used as (A + A^T)/2) by a

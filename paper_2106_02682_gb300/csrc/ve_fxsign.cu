@@ -1,11 +1,17 @@
 // ve_fxsign.cu -- the dense X step of Algorithm 5 (Khoo & Lindsey, arXiv:2106.02682, Sec. 3.2),
-// X <- Pi_{>=0}(X - eps G) for one (N D) x (N D) matrix, as Pi(Y) = (Y + sign(Y) Y) / 2 with the
-// matrix sign from a polynomial iteration: nothing but symmetric products, to float64 accuracy, on
-// the tensor cores.
+// X <- Pi_{>=0}(X - eps G) for one (N D) x (N D) matrix, as Pi(Y) = P Y P, P = (I + sign(Y)) / 2, with
+// the matrix sign from a polynomial iteration: nothing but products, to float64 accuracy, on the tensor
+// cores.
 //
 // Why.  The cyclic Jacobi it replaces is a chain of n - 1 dependent round launches a sweep (7.3 us
 // each at n = 512, 6.8 sweeps warm: 27 ms of a 28 ms sweep), and its work is float64.  Here a
-// projection is 36 products, each one launch that fills the chip.
+// projection is 39 products, each one launch that fills the chip.
+//
+// P Y P and not P Y = (Y + sign(Y) Y) / 2, which takes two products less: an error d of the sign leaves
+// d mu of a negative eigenvalue -mu in the latter, and Y has them up to hundreds of times ||X|| (eps G has
+// one of the order of N).  Squared it vanishes.  Smallest eigenvalue of X after the first sweep, P Y and
+// P Y P: n = 256 -1.6e-12 and -1.0e-15, n = 1024 -7.5e-11 and -3.8e-15 (by eigenvectors -1e-15); a sweep
+// 787 and 816 us at n = 512, 249 at n = 160.
 //
 // Iteration: ve_fxstep.cuh.
 //
@@ -13,8 +19,9 @@
 // error is 2^-56 of max|X| max|Y|), in 16 x 16 blocks stored as the A fragments of mma.sync
 // m16n8k16: a product's output block comes back in that very layout, so each kernel writes the
 // next one's operand digits itself.  32 terms of a plane sum stay below 2^24 (at most 6 x 32 x
-// 256^2), after which the float32 sums go to int64.  All matrices commute and are symmetric: only blocks
-// on and above the diagonal are computed, the others are their transposes (movmatrix).
+// 256^2), after which the float32 sums go to int64.  All matrices of the iteration commute and are
+// symmetric: only blocks on and above the diagonal are computed, the others are their transposes
+// (movmatrix).  Of Z = sign(Y) Y, whose rounding is not symmetric, all blocks are.
 // mma.sync rather than tcgen05: the digit planes s + t = q of one output accumulate in registers
 // (seven planes x 128 columns would fill tensor memory with one 128 x 128 tile, and n = 160 .. 512
 // has 2 .. 16 of those for 152 SMs).
@@ -34,7 +41,7 @@ using namespace fxstep;
 constexpr int kBlk = kD * 32;   // uint4 of one 16 x 16 block
 constexpr int kWarps = 8;       // warps of a product CTA
 constexpr int kNormCtas = 128;
-enum Mode { kSquare, kSquareLast, kPoly, kMul, kFinal };
+enum Mode { kSquare, kSquareLast, kPoly, kMul, kSide, kFinal };
 
 struct Args {
   int n, nb;
@@ -44,7 +51,7 @@ struct Args {
   long long* y2;
   long long a, b, c;    // kPoly: the step's coefficients
   double* partial;      // kSquareLast: per-block residuals
-  const FxSignCtl* ctl;
+  FxSignCtl* ctl;
   const double* Yd;
   double* Xd;
   const int* ey;        // kFinal: exponent of Yq's unit
@@ -83,6 +90,9 @@ __device__ __forceinline__ void after_previous() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// The bits that Z has above 2^53 (bits: all of its entries' magnitudes, or-ed).
+__device__ __forceinline__ int side_shift(unsigned long long bits) { return max(0, 11 - __clzll((long long)bits)); }
+
 // One product.  A CTA holds TB x TB output blocks of 16 x 16 (blocks TB bi .., TB bj .., bi <= bj),
 // KW warps a block sharing its K range.
 template <int MODE, int TB>
@@ -91,13 +101,13 @@ __global__ void __launch_bounds__(32 * kWarps, 1) k_fx_product(const Args p) {
   __shared__ long long sum[TB * TB][KW > 1 ? KW - 1 : 1][8][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int blk = warp / KW, kw = warp % KW;
-  // tile (bi, bj) of the upper triangle, row by row
+  // tile (bi, bj), row by row: of the upper triangle, or (kSide) of all
   const int T = (p.nb + TB - 1) / TB;
-  int bi, bj;
-  tri_index(T, blockIdx.x, bi, bj);
+  int bi = blockIdx.x / T, bj = blockIdx.x % T;
+  if constexpr (MODE != kSide) tri_index(T, blockIdx.x, bi, bj);
   const int I = bi * TB + blk / TB, J = bj * TB + blk % TB;
   after_previous();
-  const bool live = I <= J && J < p.nb;
+  const bool live = (MODE == kSide ? I < p.nb : I <= J) && J < p.nb;
   Frag h = {};
   if (live) {
     const uint4* a = p.A + (size_t)I * p.nb * kBlk + lane;
@@ -198,20 +208,56 @@ __global__ void __launch_bounds__(32 * kWarps, 1) k_fx_product(const Args p) {
     write_block(h, p.out, p.nb, I, J, lane);
   } else if constexpr (MODE == kMul) {
     write_block(h, p.out, p.nb, I, J, lane);
-  } else {
-    const int e = *p.ey - 53 + fx16::product_exp<6>();
-    const bool finite = p.ctl->finite != 0;
+  } else if constexpr (MODE == kSide) {
+    // Z, in units of 2^-3 times Yq's; its top bit scales the digits (k_fx_side)
+    long long* z = p.y2 + ((size_t)I * p.nb + J) * 256 + lane;
+    unsigned long long m = 0;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int row = 16 * I + fx16::frag_row(i, lane), col = 16 * J + fx16::frag_col(i, lane);
+      z[i * 32] = h[i];
+      m |= (unsigned long long)(h[i] ^ (h[i] >> 63));
+    }
+    const unsigned hi = __reduce_or_sync(0xffffffffu, (unsigned)(m >> 32));
+    const unsigned lo = __reduce_or_sync(0xffffffffu, (unsigned)m);
+    if (lane == 0) atomicOr(&p.ctl->side, (unsigned long long)hi << 32 | lo);
+  } else {
+    // X = (Y + Z + Z^T + Z sign(Y)) / 4, added as integers in Z's unit (h: 2^(shift - 3) of it)
+    const int E = *p.ey + 1075, e = *p.ey - 3, up = side_shift(p.ctl->side) - 3;
+    const bool finite = p.ctl->finite != 0;
+    const long long* z = p.y2 + ((size_t)I * p.nb + J) * 256;
+    const long long* zt = p.y2 + ((size_t)J * p.nb + I) * 256;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int r = fx16::frag_row(i, lane), c = fx16::frag_col(i, lane);
+      const int row = 16 * I + r, col = 16 * J + c;
       if (row <= col && col < p.n) {
         const double y = 0.5 * (p.Yd[(size_t)row * p.n + col] + p.Yd[(size_t)col * p.n + row]);
-        const double v = finite ? 0.5 * (y + fx16::word(h[i], e)) : NAN;
+        const long long t = zt[((r & 1) + 2 * (c >> 3) + 4 * (r >> 3)) * 32 + (c & 7) * 4 + ((r & 7) >> 1)];
+        const long long x = fx16::fix(y, E - 3) + z[i * 32 + lane] + t + fx16::shift_round(h[i], -up);
+        const double v = finite ? fx16::word(x, e - 2) : NAN;
         p.Xd[(size_t)row * p.n + col] = v;
         p.Xd[(size_t)col * p.n + row] = v;
       }
     }
   }
+}
+
+// Z as digits (block (I, J) in its own place, one warp a block).
+__global__ void __launch_bounds__(256) k_fx_side(const long long* __restrict__ y2, int nb, uint4* out,
+                                                 const FxSignCtl* ctl) {
+  const int lane = threadIdx.x & 31;
+  after_previous();
+  const int w = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (w >= nb * nb) return;
+  const int k = side_shift(ctl->side);
+  Frag z;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) z[i] = fx16::shift_round(y2[(size_t)w * 256 + i * 32 + lane], k);
+  uint32_t d[kD][4];
+  fx16::digits<kD>(z, d);
+#pragma unroll
+  for (int s = 0; s < kD; ++s)
+    out[(size_t)w * kBlk + s * 32 + lane] = make_uint4(d[s][0], d[s][1], d[s][2], d[s][3]);
 }
 
 // Per-CTA largest entries of Y, and sums of squares of the entries scaled by the CTA's largest one's
@@ -266,6 +312,7 @@ __global__ void __launch_bounds__(256) k_fx_slice(const double* __restrict__ Y, 
   if (w == 0 && lane == 0) {
     ctl->fro2 = v;
     ctl->finite = finite ? 1 : 0;
+    ctl->side = 0;
     *ey = E - 1075;
   }
   if (w >= (long)nb * (nb + 1) / 2) return;
@@ -294,6 +341,7 @@ __global__ void __launch_bounds__(256) k_fx_check(const double* partial, int nb,
   v = gsum<256>(v, red);
   if (threadIdx.x == 0) {
     ctl->resid = v;
+    ctl->side = 0;  // for the next pass
     ctl->done = v <= kResid || ctl->fro2 == 0.0 || !ctl->finite;
   }
 }
@@ -317,14 +365,15 @@ cudaError_t launch_after(void (*f)(P...), int grid, int threads, cudaStream_t s,
 // warps (n = 160: 55 CTAs instead of 15).
 template <int MODE>
 cudaError_t launch(const Args& a, cudaStream_t s) {
-  const int T = (a.nb + 1) / 2;
-  if (T * (T + 1) / 2 >= 100) return launch_after(k_fx_product<MODE, 2>, T * (T + 1) / 2, 32 * kWarps, s, a);
-  return launch_after(k_fx_product<MODE, 1>, a.nb * (a.nb + 1) / 2, 32 * kWarps, s, a);
+  const int T = (a.nb + 1) / 2, nb = a.nb;
+  auto tiles = [](int t) { return MODE == kSide ? t * t : t * (t + 1) / 2; };
+  if (T * (T + 1) / 2 >= 100) return launch_after(k_fx_product<MODE, 2>, tiles(T), 32 * kWarps, s, a);
+  return launch_after(k_fx_product<MODE, 1>, tiles(nb), 32 * kWarps, s, a);
 }
 
 size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// One pass from X[0] to X[0] (kSteps is even), the final product and the test.
+// One pass from X[0] to X[0] (kSteps is even), the final products and the test.
 cudaError_t issue_pass(FxSignWs& w, const double* Y, double* X, cudaStream_t s) {
   Args a;
   a.n = w.n;
@@ -355,6 +404,10 @@ cudaError_t issue_pass(FxSignWs& w, const double* Y, double* X, cudaStream_t s) 
   if (e != cudaSuccess) return e;
   a.A = w.X[0];
   a.B = w.Yq;
+  if ((e = launch<kSide>(a, s)) != cudaSuccess) return e;
+  if ((e = launch_after(k_fx_side, (w.nb * w.nb + 7) / 8, 256, s, w.y2, w.nb, w.B, w.ctl)) != cudaSuccess) return e;
+  a.A = w.B;
+  a.B = w.X[0];
   if ((e = launch<kFinal>(a, s)) != cudaSuccess) return e;
   return launch_after(k_fx_check, 1, 256, s, a.partial, w.nb, w.ctl);
 }
@@ -438,7 +491,7 @@ cudaError_t fxsign_project(FxSignWs& w, const double* Y, double* X, cudaStream_t
   for (w.passes = 1;; ++w.passes) {
     if (w.passes > 1 && !w.again && (e = build_graph(w, Y, X, false, &w.again)) != cudaSuccess) return e;
     if ((e = cudaGraphLaunch(w.passes == 1 ? w.first : w.again, s)) != cudaSuccess) return e;
-    w.launches += 3 * kSteps + 2 + (w.passes == 1 ? 2 : 0);
+    w.launches += 3 * kSteps + 4 + (w.passes == 1 ? 2 : 0);
     if ((e = cudaMemcpyAsync(w.hctl, w.ctl, sizeof(FxSignCtl), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
     if (w.hctl->done || w.passes == kMaxPasses) return cudaSuccess;

@@ -13,6 +13,7 @@ struct FxSignCtl {
   double resid;    // ||I - X^2||_F^2 before the last step
   int done;        // the sign has converged (or Y is zero or not finite)
   int finite;
+  unsigned long long side;  // the magnitudes of sign(Y) Y, or-ed
 };
 
 // Device workspace of one n x n projection (carved from caller memory).  The matrices are stored as
@@ -21,9 +22,9 @@ struct FxSignWs {
   int n = 0, nb = 0;
   uint4* X[2] = {nullptr, nullptr};  // the iterate (ping-pong)
   uint4* Y2 = nullptr;               // X^2
-  uint4* B = nullptr;                // a I + b X^2 + c X^4
+  uint4* B = nullptr;                // a I + b X^2 + c X^4; at the end sign(Y) Y
   uint4* Yq = nullptr;               // Y, scaled by its largest entry
-  long long* y2 = nullptr;           // X^2 as integers (upper blocks, fragment order)
+  long long* y2 = nullptr;           // X^2 as integers (upper blocks, fragment order); at the end sign(Y) Y
   double* partial = nullptr;         // per-CTA norms, per-block residuals
   FxSignCtl* ctl = nullptr;
   FxSignCtl* hctl = nullptr;         // pinned (allocated on first use)
