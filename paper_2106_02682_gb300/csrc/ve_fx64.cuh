@@ -1,9 +1,10 @@
 // ve_fx64.cuh -- PSD projection of one 64 x 64 matrix (real symmetric or complex Hermitian) by one
-// CTA, to float64 accuracy without float64 products: Pi(C) = (C + sign(C) C) / 2 with the matrix
-// sign iteration of ve_fxstep.cuh and the sliced fixed-point products of ve_fx16.cuh.
+// CTA, to float64 accuracy without float64 products: Pi(C) = P C P, P = (I + sign(C)) / 2, with the matrix
+// sign iteration of ve_fxstep.cuh and the sliced fixed-point products of ve_fx16.cuh (P from both sides:
+// ve_fxsign.cu).
 //
 // Why the sign and not eigenvectors, as at 16 x 16: a float32 Jacobi sweep of a 64 x 64 matrix is 63
-// rounds of CTA barriers, so the eigensolve would cost more than the 37 products of the iteration,
+// rounds of CTA barriers, so the eigensolve would cost more than the 39 products of the iteration,
 // which need no starting vectors and no store either.
 //
 // Ten warps own the ten 16 x 16 blocks on and above the diagonal (the others are their conjugate
@@ -63,7 +64,41 @@ __device__ __forceinline__ void write_block(const Frag& zr, const Frag& zi, uint
   }
 }
 
-// Block (I, J) of A B for commuting Hermitian A, B: sum_k A_Ik conj(B_Jk)^T.
+// The digits of block (I, J) of any matrix.
+template <bool CPLX>
+__device__ __forceinline__ void write_one(const Frag& zr, const Frag& zi, uint4* out, int I, int J, int lane) {
+#pragma unroll
+  for (int part = 0; part < (CPLX ? 2 : 1); ++part) {
+    uint32_t d[kD][4];
+    fx16::digits<kD>(part ? zi : zr, d);
+    uint4* o = out + part * kPart + (I * 4 + J) * (kD * 32) + lane;
+#pragma unroll
+    for (int s = 0; s < kD; ++s) o[s * 32] = make_uint4(d[s][0], d[s][1], d[s][2], d[s][3]);
+  }
+}
+
+// x += the transpose of t, 16 bits of its words at a time.
+__device__ __forceinline__ void add_transpose(Frag& x, const Frag& t, bool negative) {
+#pragma unroll
+  for (int a = 0; a < 2; ++a)  // row half a, column half b of t
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const unsigned long long t0 = (unsigned long long)t[2 * a + 4 * b], t1 = (unsigned long long)t[2 * a + 4 * b + 1];
+      unsigned long long v0 = 0, v1 = 0;
+#pragma unroll
+      for (int s = 0; s < 64; s += 16) {
+        const uint32_t u = (uint32_t)((t0 >> s) & 0xffff) | ((uint32_t)((t1 >> s) & 0xffff) << 16);
+        const uint32_t v = fxstep::transpose8(u);
+        v0 |= (unsigned long long)(v & 0xffff) << s;
+        v1 |= (unsigned long long)(v >> 16) << s;
+      }
+      long long &x0 = x[2 * b + 4 * a], &x1 = x[2 * b + 4 * a + 1];
+      x0 += negative ? -(long long)v0 : (long long)v0;
+      x1 += negative ? -(long long)v1 : (long long)v1;
+    }
+}
+
+// Block (I, J) of A B, B Hermitian: sum_k A_Ik conj(B_Jk)^T.
 template <bool CPLX>
 __device__ __forceinline__ void product(const uint4* A, const uint4* B, int I, int J, Frag& zr, Frag& zi, int lane) {
 #pragma unroll 1
@@ -254,7 +289,8 @@ __device__ int project(unsigned char* sm, int tid, Load load, Store store) {
         __syncthreads();
       }
     }
-    // C scaled by its largest entry's binade: sign(C) C
+    // Z = sign(C) C, all blocks (its rounding is not Hermitian), C scaled by its largest entry's binade:
+    // units of 2^-3 times C's
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       double re, im;
@@ -264,19 +300,61 @@ __device__ int project(unsigned char* sm, int tid, Load load, Store store) {
     }
     write_block<CPLX>(hr, hi, Z, I, J, lane);
     __syncthreads();
+    Frag tr, ti;
     product<CPLX>(X, Z, I, J, hr, hi, lane);
+    if (I != J) product<CPLX>(X, Z, J, I, tr, ti, lane);
+    int top = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      if (I == J) {
+        tr[i] = hr[i];
+        if constexpr (CPLX) ti[i] = hi[i];
+      }
+      unsigned long long m = (unsigned long long)(hr[i] ^ (hr[i] >> 63)) | (unsigned long long)(tr[i] ^ (tr[i] >> 63));
+      if constexpr (CPLX)
+        m |= (unsigned long long)(hi[i] ^ (hi[i] >> 63)) | (unsigned long long)(ti[i] ^ (ti[i] >> 63));
+      top = max(top, 64 - __clzll((long long)m));
+    }
+    const int k = max(0, reduce_max(top, red, tid) - 53);  // digits hold 53 bits
+    {
+      Frag qr, qi;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        qr[i] = fx16::shift_round(hr[i], k);
+        if constexpr (CPLX) qi[i] = fx16::shift_round(hi[i], k);
+      }
+      write_one<CPLX>(qr, qi, Z, I, J, lane);
+      if (I != J) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          qr[i] = fx16::shift_round(tr[i], k);
+          if constexpr (CPLX) qi[i] = fx16::shift_round(ti[i], k);
+        }
+        write_one<CPLX>(qr, qi, Z, J, I, lane);
+      }
+    }
+    add_transpose(hr, tr, false);
+    if constexpr (CPLX) add_transpose(hi, ti, true);
+    __syncthreads();
+    // C + Z + Z^H + Z sign(C), four times the result, in Z's units
+    product<CPLX>(Z, X, I, J, tr, ti, lane);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      double re, im;
+      entry(i, re, im);
+      hr[i] += fx16::fix(re, E - 3) + fx16::shift_round(tr[i], 3 - k);
+      if constexpr (CPLX) hi[i] += fx16::fix(im, E - 3) + fx16::shift_round(ti[i], 3 - k);
+    }
   } else {
 #pragma unroll
     for (int i = 0; i < 8; ++i) hr[i] = hi[i] = 0;
   }
-  const int e = E - 1075 - 53 + fx16::product_exp<6>();
+  const int e = E - 1075 - 53 + fx16::product_exp<6>() - 2;
   double re[8], im[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    double cr, ci;
-    entry(i, cr, ci);
-    re[i] = finite ? 0.5 * (cr + fx16::word(hr[i], e)) : NAN;
-    im[i] = !CPLX || row(i) == col(i) ? 0.0 : finite ? 0.5 * (ci + fx16::word(hi[i], e)) : NAN;
+    re[i] = finite ? fx16::word(hr[i], e) : NAN;
+    im[i] = !CPLX || row(i) == col(i) ? 0.0 : finite ? fx16::word(hi[i], e) : NAN;
   }
   __syncthreads();
 #pragma unroll
