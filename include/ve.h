@@ -414,8 +414,10 @@ int ve_general_get_status(ve_general* h, ve_status* out);
  * raw_bound = sum_i lmin(K_i) + sum_{i<j} lmin(K_ij), K_ij = H'_ij + A1^* Lambda1_ij +
  * A2^* Lambda2_ij, K_i = H'_i - sum_{j>i} Lambda1_ij - sum_{j<i} Lambda2_ji; x_min_eig =
  * lmin(X); x_neg_correction = N m max(0, -x_min_eig); bound_per_spin = (raw_bound -
- * x_neg_correction) / nspins.  All in float64 on the GPU.  The eigensolve of X (cyclic Jacobi over
- * the whole GPU) starts from the eigenvectors of the handle's last bound.  Synchronous. */
+ * x_neg_correction) / nspins.  Everything to float64 accuracy on the GPU.  x_min_eig is a lower bound on
+ * lmin(X) up to rounding, within (N D) 2^-53 ||X||_F of it: -4 ||(I - P) X (I - P)||_2 at most where X is
+ * singular to rounding, as after an X step, else from an eigensolve of X (cyclic Jacobi over the whole GPU,
+ * which starts from the eigenvectors of the handle's last one).  Synchronous. */
 int ve_general_bound(ve_general* h, ve_cert* out);
 
 /* Packed state: rho_i (N m^2), rho~ (K D^2), Lambda (K D^2), Lambda1 (K m^2), Lambda2 (K m^2),

@@ -54,7 +54,7 @@ struct Args {
   FxSignCtl* ctl;
   const double* Yd;
   double* Xd;
-  const int* ey;        // kFinal: exponent of Yq's unit
+  int sg;               // kFinal: 1 for P Y P, -1 for (I - P) Y (I - P)
 };
 
 // Digits of the integers z as block (I, J), and transposed as block (J, I).  Of a diagonal block the
@@ -221,8 +221,8 @@ __global__ void __launch_bounds__(32 * kWarps, 1) k_fx_product(const Args p) {
     const unsigned lo = __reduce_or_sync(0xffffffffu, (unsigned)m);
     if (lane == 0) atomicOr(&p.ctl->side, (unsigned long long)hi << 32 | lo);
   } else {
-    // X = (Y + Z + Z^T + Z sign(Y)) / 4, added as integers in Z's unit (h: 2^(shift - 3) of it)
-    const int E = *p.ey + 1075, e = *p.ey - 3, up = side_shift(p.ctl->side) - 3;
+    // X = (Y +- (Z + Z^T) + Z sign(Y)) / 4, added as integers in Z's unit (h: 2^(shift - 3) of it)
+    const int E = p.ctl->ey + 1075, e = p.ctl->ey - 3, up = side_shift(p.ctl->side) - 3;
     const bool finite = p.ctl->finite != 0;
     const long long* z = p.y2 + ((size_t)I * p.nb + J) * 256;
     const long long* zt = p.y2 + ((size_t)J * p.nb + I) * 256;
@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(32 * kWarps, 1) k_fx_product(const Args p) {
       if (row <= col && col < p.n) {
         const double y = 0.5 * (p.Yd[(size_t)row * p.n + col] + p.Yd[(size_t)col * p.n + row]);
         const long long t = zt[((r & 1) + 2 * (c >> 3) + 4 * (r >> 3)) * 32 + (c & 7) * 4 + ((r & 7) >> 1)];
-        const long long x = fx16::fix(y, E - 3) + z[i * 32 + lane] + t + fx16::shift_round(h[i], -up);
+        const long long x = fx16::fix(y, E - 3) + p.sg * (z[i * 32 + lane] + t) + fx16::shift_round(h[i], -up);
         const double v = finite ? fx16::word(x, e - 2) : NAN;
         p.Xd[(size_t)row * p.n + col] = v;
         p.Xd[(size_t)col * p.n + row] = v;
@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(256) k_fx_norm(const double* __restrict__ Y, i
 // X_0 = Y / ||Y||_F and Y scaled by its largest entry, as digits; one warp a block on or above the
 // diagonal.  Every warp adds the norms up itself, in one order.
 __global__ void __launch_bounds__(256) k_fx_slice(const double* __restrict__ Y, int n, int nb, const double* partial,
-                                                  uint4* X, uint4* Yq, FxSignCtl* ctl, int* ey) {
+                                                  uint4* X, uint4* Yq, FxSignCtl* ctl) {
   const int lane = threadIdx.x & 31;
   after_previous();
   double v = 0.0, m = 0.0;
@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(256) k_fx_slice(const double* __restrict__ Y, 
     ctl->fro2 = v;
     ctl->finite = finite ? 1 : 0;
     ctl->side = 0;
-    *ey = E - 1075;
+    ctl->ey = E - 1075;
   }
   if (w >= (long)nb * (nb + 1) / 2) return;
   int I, J;
@@ -346,6 +346,45 @@ __global__ void __launch_bounds__(256) k_fx_check(const double* partial, int nb,
   }
 }
 
+// ||X^2||_F^2 of the integers of X^2 (upper blocks), in a fixed order.
+__global__ void __launch_bounds__(1024) k_fx_fro(const long long* __restrict__ y2, int nb, FxSignCtl* ctl) {
+  __shared__ double red[32];
+  after_previous();
+  double v = 0.0;
+  for (int b = threadIdx.x >> 8; b < nb * nb; b += 4) {
+    const int I = b / nb, J = b % nb;
+    if (I > J) continue;
+    const double x = (double)y2[(size_t)b * 256 + (threadIdx.x & 255)] * 1.1102230246251565e-16;
+    v = fma(I == J ? x : 2.0 * x, x, v);
+  }
+  v = gsum<1024>(v, red);
+  if (threadIdx.x == 0) ctl->resid = v;
+}
+
+// The smallest eigenvalue of a matrix of up to 16 rows by one warp (fx16::lowest; rows past n decoupled,
+// with the largest entry on their diagonal, which is no smaller) into ctl->resid.
+__global__ void __launch_bounds__(32) k_fx_small(const double* __restrict__ Y, int n, FxSignCtl* ctl) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x;
+  double c[8], m = 0.0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int row = fx16::frag_row(i, lane), col = fx16::frag_col(i, lane);
+    c[i] = row < n && col < n ? 0.5 * (Y[row * n + col] + Y[col * n + row]) : 0.0;
+    m = fmax(m, fabs(c[i]));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, shfl_xor(m, o));
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    if (fx16::frag_row(i, lane) == fx16::frag_col(i, lane) && fx16::frag_row(i, lane) >= n) c[i] = m;
+  Frag q, none;
+  int e = 0;
+  double v = NAN;
+  if (fx16::fix_matrix<false>(c, c, q, none, e)) v = fx16::lowest<false>(q, none, e, smem_raw, lane);
+  if (lane == 0) ctl->resid = v;
+}
+
 // A launch that need not wait for the one before it on the stream to finish (after_previous).
 template <class... P, class... A>
 cudaError_t launch_after(void (*f)(P...), int grid, int threads, cudaStream_t s, A... args) {
@@ -374,8 +413,9 @@ cudaError_t launch(const Args& a, cudaStream_t s) {
 size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // One pass from X[0] to X[0] (kSteps is even), the final products and the test.
-cudaError_t issue_pass(FxSignWs& w, const double* Y, double* X, cudaStream_t s) {
+cudaError_t issue_pass(FxSignWs& w, const double* Y, double* X, int sg, cudaStream_t s) {
   Args a;
+  a.sg = sg;
   a.n = w.n;
   a.nb = w.nb;
   a.y2 = w.y2;
@@ -383,7 +423,6 @@ cudaError_t issue_pass(FxSignWs& w, const double* Y, double* X, cudaStream_t s) 
   a.ctl = w.ctl;
   a.Yd = Y;
   a.Xd = X;
-  a.ey = reinterpret_cast<const int*>(w.ctl + 1);
   cudaError_t e = cudaSuccess;
   for (int k = 0; k < kSteps && e == cudaSuccess; ++k) {
     a.A = a.B = w.X[k & 1];
@@ -423,10 +462,9 @@ cudaError_t build_graph(FxSignWs& w, const double* Y, double* X, bool first, cud
       const int blocks = w.nb * (w.nb + 1) / 2;
       e = cudaGetLastError();
       if (e == cudaSuccess)
-        e = launch_after(k_fx_slice, (blocks + 7) / 8, 256, cs, Y, w.n, w.nb, w.partial, w.X[0], w.Yq, w.ctl,
-                         reinterpret_cast<int*>(w.ctl + 1));
+        e = launch_after(k_fx_slice, (blocks + 7) / 8, 256, cs, Y, w.n, w.nb, w.partial, w.X[0], w.Yq, w.ctl);
     }
-    if (e == cudaSuccess) e = issue_pass(w, Y, X, cs);
+    if (e == cudaSuccess) e = issue_pass(w, Y, X, 1, cs);
     cudaGraph_t g = nullptr;
     const cudaError_t e2 = cudaStreamEndCapture(cs, &g);
     if (e == cudaSuccess) e = e2;
@@ -437,13 +475,23 @@ cudaError_t build_graph(FxSignWs& w, const double* Y, double* X, bool first, cud
   return e;
 }
 
+cudaError_t host_ctl(FxSignWs& w) {
+  return w.hctl ? cudaSuccess : cudaMallocHost((void**)&w.hctl, 2 * sizeof(FxSignCtl));
+}
+
+// The root of a scaled sum of squares (FxSignCtl::fro2).
+double unscaled(double sum, int ey) {
+  const int E = ey + 1075;
+  return ldexp(sqrt(sum), E < 2045 ? E - 1023 : 1022);
+}
+
 }  // namespace
 
 size_t fxsign_ws_bytes(int n) {
   if (n < 2 || (n & 1)) return 0;
   const size_t nb = (n + 15) / 16;
   return 5 * al256(nb * nb * kBlk * sizeof(uint4)) + al256(nb * nb * 256 * sizeof(long long)) +
-         al256((2 * kNormCtas + nb * nb) * sizeof(double)) + al256(sizeof(FxSignCtl) + sizeof(int));
+         al256((2 * kNormCtas + nb * nb) * sizeof(double)) + al256(2 * sizeof(FxSignCtl));
 }
 
 int fxsign_ws_init(FxSignWs& w, int n, void* mem, size_t bytes) {
@@ -477,7 +525,7 @@ void fxsign_ws_release(FxSignWs& w) {
 
 cudaError_t fxsign_project(FxSignWs& w, const double* Y, double* X, cudaStream_t s) {
   cudaError_t e;
-  if (!w.hctl && (e = cudaMallocHost((void**)&w.hctl, sizeof(FxSignCtl))) != cudaSuccess) return e;
+  if ((e = host_ctl(w)) != cudaSuccess) return e;
   if (w.first && (w.Yd != Y || w.Xd != X)) {
     cudaGraphExecDestroy(w.first);
     if (w.again) cudaGraphExecDestroy(w.again);
@@ -495,6 +543,64 @@ cudaError_t fxsign_project(FxSignWs& w, const double* Y, double* X, cudaStream_t
     if ((e = cudaMemcpyAsync(w.hctl, w.ctl, sizeof(FxSignCtl), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
     if (w.hctl->done || w.passes == kMaxPasses) return cudaSuccess;
+  }
+}
+
+// M = N Y N, N = (I - sign(Y)) / 2, is zero but for rounding and the eigenvalues whose sign is not
+// resolved (s near 0: M has a quarter of them) or is negative (all of them), so lmin(Y) >= -4 ||M||_2 up to
+// rounding; ||M||_2 <= ||M^2||_F^(1/2), four to five times less than ||M||_F where M is rounding.  One
+// pass is enough where Y has no eigenvalue between rounding and 3e-6 ||Y||_F.  An unresolved sign
+// (||I - S^2||_F^2 >= 1/2) and a small bound say that lmin(Y) is zero to rounding.
+// Measured, a general bound after 60 sweeps (eigensolve of X warm from the X step's own eigenvectors / from
+// the last bound's / here): n = 24 767 / 1198 / 228 us, n = 160 3.4 / 8.6 / 0.45 ms, n = 512 8.7 / 60 /
+// 1.26 ms, n = 1024 42 / 309 / 6.5 ms; the bounds -1.1e-14 / -1.5e-12 / -1.1e-14 at n = 512.
+cudaError_t fxsign_lmin(FxSignWs& w, const double* Y, double* scratch, cudaStream_t s, double* lmin, bool* found) {
+  cudaError_t e;
+  if ((e = host_ctl(w)) != cudaSuccess) return e;
+  FxSignCtl* h = w.hctl;
+  auto read = [&]() {
+    const cudaError_t r = cudaMemcpyAsync(h, w.ctl, 2 * sizeof(FxSignCtl), cudaMemcpyDeviceToHost, s);
+    return r != cudaSuccess ? r : cudaStreamSynchronize(s);
+  };
+  *found = true;
+  if (w.n <= 16) {  // by eigenvalues: one launch, not 47 (a bound at n = 8: 105 to 145 us)
+    k_fx_small<<<1, 32, fx16::Smem<false>::bytes + fx16::Smem<false>::vectors, s>>>(Y, w.n, w.ctl);
+    if ((e = cudaGetLastError()) != cudaSuccess || (e = read()) != cudaSuccess) return e;
+    *lmin = h[0].resid;
+    return cudaSuccess;
+  }
+  const int slices = (w.nb * (w.nb + 1) / 2 + 7) / 8;
+  auto slice = [&](const double* from, uint4* x, uint4* q, FxSignCtl* ctl) {
+    k_fx_norm<<<kNormCtas, 256, 0, s>>>(from, w.n, w.partial);
+    const cudaError_t r = cudaGetLastError();
+    return r != cudaSuccess ? r : launch_after(k_fx_slice, slices, 256, s, from, w.n, w.nb, w.partial, x, q, ctl);
+  };
+  if ((e = slice(Y, w.X[0], w.Yq, w.ctl)) != cudaSuccess) return e;
+  for (int pass = 1;; ++pass) {
+    if ((e = issue_pass(w, Y, scratch, -1, s)) != cudaSuccess) return e;
+    if ((e = slice(scratch, w.Y2, w.B, w.ctl + 1)) != cudaSuccess) return e;
+    Args a = {};
+    a.n = w.n;
+    a.nb = w.nb;
+    a.A = a.B = w.Y2;
+    a.out = w.B;
+    a.y2 = w.y2;
+    if ((e = launch<kSquare>(a, s)) != cudaSuccess) return e;
+    if ((e = launch_after(k_fx_fro, 1, 1024, s, w.y2, w.nb, w.ctl + 1)) != cudaSuccess) return e;
+    if ((e = read()) != cudaSuccess) return e;
+    if (!h[0].finite) {
+      *lmin = NAN;
+      return cudaSuccess;
+    }
+    const double b = 4.0001 * unscaled(h[1].fro2 * sqrt(h[1].resid), h[1].ey);
+    if (h[0].resid >= 0.5 && b <= w.n * 1.1102230246251565e-16 * unscaled(h[0].fro2, h[0].ey)) {
+      *lmin = 0.0 - b;
+      return cudaSuccess;
+    }
+    if (h[0].done || pass == kMaxPasses) {
+      *found = false;
+      return cudaSuccess;
+    }
   }
 }
 

@@ -630,7 +630,7 @@ struct ve_general {
   GenStatus *dst = nullptr, *hst = nullptr;
   FxSignWs sws;      // the X step (ve_fxsign.cu)
   DenseWs bws;       // the bound's eigensolve of X
-  long bounds = 0;   // of those so far (each starts from the eigenvectors of the one before)
+  long bounds = 0;   // eigensolves so far (each starts from the eigenvectors of the one before)
   bool pair_warm = false;
   int fermionic = 0;
   // profiling: 0 pair pass, 1 cluster + dual + status, 2 dense eigensolve, 3 reconstruction
@@ -660,7 +660,7 @@ struct Guard {
   }
 };
 
-// Every refresh-th bound restarts its eigensolve of X from V = I, so that rounding in the rotated
+// Every refresh-th eigensolve of X restarts from V = I, so that rounding in the rotated
 // eigenvectors cannot accumulate.
 constexpr long kRefresh = 256;
 
@@ -1156,28 +1156,34 @@ int ve_general_bound(ve_general* h, ve_cert* out) {
   GenArgs a = gen_args(h);
   VG_CU(launch_gbound_pair(a, h->lmin_p, s));
   VG_CU(launch_small(a, 2, h->lmin_c, s));
-  // lmin(X): the eigensolve starts from the last bound's eigenvectors
-  // (from V = I again after one that did not end in a finite bound: its eigenvectors may not be)
-  const int mode = h->bounds % kRefresh ? DENSE_WARM : DENSE_COLD;
+  // lmin(X): zero to rounding after an X step (fxsign_lmin; Y is free between sweeps).  Else by an
+  // eigensolve, which starts from the eigenvectors of the last one (from V = I again after one that did
+  // not end in a finite bound: its eigenvectors may not be)
+  double xmin = 0.0;
+  bool found = false;
+  VG_CU(fxsign_lmin(h->sws, h->X, h->Y, s, &xmin, &found));
   const long next = h->bounds + 1;
-  h->bounds = 0;
-  VG_CU(dense_eig(h->bws, h->X, mode, s));
-  VG_CU(dense_lmin_certified(h->bws, s));
+  if (!found) {
+    const int mode = h->bounds % kRefresh ? DENSE_WARM : DENSE_COLD;
+    h->bounds = 0;
+    VG_CU(dense_eig(h->bws, h->X, mode, s));
+    VG_CU(dense_lmin_certified(h->bws, s));
+  }
   std::vector<double> lp((size_t)h->K), lc((size_t)h->N);
   DenseCtl ctl;
   VG_CU(cudaMemcpyAsync(lp.data(), h->lmin_p, lp.size() * 8, cudaMemcpyDeviceToHost, s));
   VG_CU(cudaMemcpyAsync(lc.data(), h->lmin_c, lc.size() * 8, cudaMemcpyDeviceToHost, s));
-  VG_CU(cudaMemcpyAsync(&ctl, h->bws.ctl, sizeof(DenseCtl), cudaMemcpyDeviceToHost, s));
+  if (!found) VG_CU(cudaMemcpyAsync(&ctl, h->bws.ctl, sizeof(DenseCtl), cudaMemcpyDeviceToHost, s));
   ve_status st;
   const int r = read_status(h, &st);  // synchronises
   if (r != VE_OK) return r;  // a non-finite iterate certifies nothing
   double raw = 0.0;
   for (double v : lc) raw += v;
   for (double v : lp) raw += v;
-  const double xmin = ctl.lmin;
+  if (!found) xmin = ctl.lmin;
   // every minimum passes a NaN on, and an Inf stays in the sum: one check covers them all
   if (!std::isfinite(raw) || !std::isfinite(xmin)) return VE_ENONFINITE;
-  h->bounds = next;
+  if (!found) h->bounds = next;
   const double corr = (double)h->N * h->m * (xmin < 0 ? -xmin : 0.0);
   out->raw_bound = raw;
   out->x_min_eig = xmin;
