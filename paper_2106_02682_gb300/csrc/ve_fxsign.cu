@@ -361,9 +361,10 @@ __global__ void __launch_bounds__(1024) k_fx_fro(const long long* __restrict__ y
   if (threadIdx.x == 0) ctl->resid = v;
 }
 
-// The smallest eigenvalue of a matrix of up to 16 rows by one warp (fx16::lowest; rows past n decoupled,
-// with the largest entry on their diagonal, which is no smaller) into ctl->resid.
-__global__ void __launch_bounds__(32) k_fx_small(const double* __restrict__ Y, int n, FxSignCtl* ctl) {
+// A matrix of up to 16 rows by one warp (ve_fx16.cuh, from V = I; rows past n decoupled, with the largest
+// entry on their diagonal, which is no smaller than its lowest eigenvalue): its projection into X, or (X
+// null) its smallest eigenvalue into ctl->resid.
+__global__ void __launch_bounds__(32) k_fx_small(const double* __restrict__ Y, int n, double* X, FxSignCtl* ctl) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x;
   double c[8], m = 0.0;
@@ -380,9 +381,35 @@ __global__ void __launch_bounds__(32) k_fx_small(const double* __restrict__ Y, i
     if (fx16::frag_row(i, lane) == fx16::frag_col(i, lane) && fx16::frag_row(i, lane) >= n) c[i] = m;
   Frag q, none;
   int e = 0;
-  double v = NAN;
-  if (fx16::fix_matrix<false>(c, c, q, none, e)) v = fx16::lowest<false>(q, none, e, smem_raw, lane);
-  if (lane == 0) ctl->resid = v;
+  const bool finite = fx16::fix_matrix<false>(c, c, q, none, e);
+  if (!X) {
+    const double v = finite ? fx16::lowest<false>(q, none, e, smem_raw, lane) : NAN;
+    if (lane == 0) ctl->resid = v;
+    return;
+  }
+  fx16::Result res = fx16::kProduct;
+  if (finite) {
+    bool dk;
+    int nsw;
+    long long* v = reinterpret_cast<long long*>(smem_raw + fx16::Smem<false>::bytes);
+    res = fx16::project<false>(q, none, e, v, false, smem_raw, lane, &dk, &nsw);
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int row = fx16::frag_row(i, lane), col = fx16::frag_col(i, lane);
+    if (row < n && col < n)
+      X[row * n + col] = !finite                  ? NAN
+                         : res == fx16::kProduct ? fx16::word(q[i], e)
+                         : res == fx16::kSame    ? c[i]
+                                                 : 0.0;
+  }
+}
+
+// n <= 16.  One launch and no test on the host, for 42 launches and a copy: a general sweep at n = 8 79 to
+// 106 us and not 157 (eigensolve over the whole GPU: 122 to 188), at n = 16 96 to 104 and not 159.
+cudaError_t small(const double* Y, int n, double* X, FxSignCtl* ctl, cudaStream_t s) {
+  k_fx_small<<<1, 32, fx16::Smem<false>::bytes + fx16::Smem<false>::vectors, s>>>(Y, n, X, ctl);
+  return cudaGetLastError();
 }
 
 // A launch that need not wait for the one before it on the stream to finish (after_previous).
@@ -524,6 +551,11 @@ void fxsign_ws_release(FxSignWs& w) {
 }
 
 cudaError_t fxsign_project(FxSignWs& w, const double* Y, double* X, cudaStream_t s) {
+  if (w.n <= 16) {
+    w.passes = 1;
+    w.launches += 1;
+    return small(Y, w.n, X, w.ctl, s);
+  }
   cudaError_t e;
   if ((e = host_ctl(w)) != cudaSuccess) return e;
   if (w.first && (w.Yd != Y || w.Xd != X)) {
@@ -564,8 +596,7 @@ cudaError_t fxsign_lmin(FxSignWs& w, const double* Y, double* scratch, cudaStrea
   };
   *found = true;
   if (w.n <= 16) {  // by eigenvalues: one launch, not 47 (a bound at n = 8: 105 to 145 us)
-    k_fx_small<<<1, 32, fx16::Smem<false>::bytes + fx16::Smem<false>::vectors, s>>>(Y, w.n, w.ctl);
-    if ((e = cudaGetLastError()) != cudaSuccess || (e = read()) != cudaSuccess) return e;
+    if ((e = small(Y, w.n, nullptr, w.ctl, s)) != cudaSuccess || (e = read()) != cudaSuccess) return e;
     *lmin = h[0].resid;
     return cudaSuccess;
   }

@@ -41,8 +41,8 @@ size_t fxsign_ws_bytes(int n);
 int fxsign_ws_init(FxSignWs& w, int n, void* mem, size_t bytes);
 void fxsign_ws_release(FxSignWs& w);
 // X <- Pi_{>=0}((Y + Y^T) / 2) (device, n x n row-major, n even; X and Y distinct).  Issues
-// everything on `s` and synchronises it once a pass (the convergence test is read on the host).  A
-// non-finite Y gives NaN throughout.  Not to be called during stream capture.
+// everything on `s` and synchronises it once a pass (the convergence test is read on the host; up to 16
+// rows there is none).  A non-finite Y gives NaN throughout.  Not to be called during stream capture.
 cudaError_t fxsign_project(FxSignWs& w, const double* Y, double* X, cudaStream_t s);
 // A lower bound on the smallest eigenvalue of (Y + Y^T) / 2 where that eigenvalue is zero to rounding, as
 // after a projection: *lmin = -4 ||N Y N||_2 at most, N = (I - sign(Y)) / 2.  *found says whether it is
