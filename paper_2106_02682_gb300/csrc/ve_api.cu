@@ -550,12 +550,13 @@ int ve_create(const ve_lattice* lattice, const ve_cluster* cluster, const ve_ham
   const size_t o_pidx = take(sizeof(int) * P);
   const size_t o_pmir = take(sizeof(int) * P);
   const size_t o_ptie = take(sizeof(int) * P);
-  const size_t o_vp64 = take(sizeof(double) * P * DD);
+  const size_t vd = D == 64 ? 0 : sizeof(double) * DD;  // 64 x 64 in float64: by the matrix sign, no vectors
+  const size_t o_vp64 = take(vd * P);
   const size_t o_vp32 = take(sizeof(float) * P * DD);
-  const size_t o_vk64 = take(sizeof(double) * 2 * N * DD);
+  const size_t o_vk64 = take(vd * 2 * N);
   const size_t o_vk32 = take(sizeof(float) * 2 * N * DD);
-  const size_t o_vpdf = take(sizeof(double) * P * DD);
-  const size_t o_vkdf = take(sizeof(double) * 2 * N * DD);
+  const size_t o_vpdf = take(vd * P);
+  const size_t o_vkdf = take(vd * 2 * N);
   const size_t o_sa = take(sizeof(double2) * N * h->plan.E);
   const size_t o_sb = take(sizeof(double2) * N * h->plan.E);
   const size_t o_tw = take(sizeof(double2) * h->plan.ntw);
@@ -600,12 +601,12 @@ int ve_create(const ve_lattice* lattice, const ve_cluster* cluster, const ve_ham
   h->pmir = (int*)(base + o_pmir);
   h->ptie = (int*)(base + o_ptie);
   h->ncanon = fft_ncanon(h->plan);
-  h->vpair[0] = base + o_vp64;
+  h->vpair[0] = vd ? base + o_vp64 : nullptr;
   h->vpair[1] = base + o_vp32;
-  h->vk[0] = base + o_vk64;
+  h->vk[0] = vd ? base + o_vk64 : nullptr;
   h->vk[1] = base + o_vk32;
-  h->vpair[2] = base + o_vpdf;
-  h->vk[2] = base + o_vkdf;
+  h->vpair[2] = vd ? base + o_vpdf : nullptr;
+  h->vk[2] = vd ? base + o_vkdf : nullptr;
   h->specA = (double2*)(base + o_sa);
   h->specB = (double2*)(base + o_sb);
   h->tw = (double2*)(base + o_tw);

@@ -63,7 +63,7 @@ struct GenArgs {
   double* a2;           // K m^2  A2 rho_ij
   double* part;         // K * 3: |rho - rho~|^2, Tr[H_ij rho_ij], Lambda1/2 feasibility terms
   double* parti;        // N: Tr[H_i rho_i]
-  double* vstore;       // K D^2: eigenvectors of the last pair projections
+  double* vstore;       // K D^2: eigenvectors of the last pair projections (D = 64: none)
   int warm;
   int fermionic;        // parity signs on the off-diagonal blocks of G and in H' (Eq. (sdpFerm))
   GenStatus* st;
@@ -1009,9 +1009,10 @@ int create_from_blocks(int N, int L, std::vector<double>& Hi, std::vector<double
   h->state_count = (size_t)N * m * m + (size_t)K * (2 * D * D + 2 * m * m) + (size_t)n * n;
   const size_t nd = (size_t)n * n;
   const size_t dense = dense_ws_bytes((int)n), sign = fxsign_ws_bytes((int)n);
+  const size_t vectors = D == 64 ? 0 : (size_t)K * D * D * 8;  // 64 x 64: by the matrix sign
   size_t bytes = al256(h->state_count * 8) + al256(Hi.size() * 8) + al256(Hij.size() * 8) +
                  2 * al256((size_t)K * m * m * 8) + al256((size_t)K * 3 * 8) + al256((size_t)N * 8) +
-                 al256(nd * 8) + al256((size_t)K * D * D * 8) + al256((size_t)K * 8) + al256((size_t)N * 8) +
+                 al256(nd * 8) + al256(vectors) + al256((size_t)K * 8) + al256((size_t)N * 8) +
                  2 * al256((size_t)K * 4) + al256(sizeof(GenStatus)) + al256(sign) + dense;
   if (cudaMalloc(&h->dev, bytes) != cudaSuccess) {
     delete h;
@@ -1037,7 +1038,7 @@ int create_from_blocks(int N, int L, std::vector<double>& Hi, std::vector<double
   h->part = (double*)take((size_t)K * 3 * 8);
   h->parti = (double*)take((size_t)N * 8);
   h->Y = (double*)take(nd * 8);
-  h->vstore = (double*)take((size_t)K * D * D * 8);
+  h->vstore = vectors ? (double*)take(vectors) : nullptr;
   h->lmin_p = (double*)take((size_t)K * 8);
   h->lmin_c = (double*)take((size_t)N * 8);
   h->pi = (int*)take((size_t)K * 4);
