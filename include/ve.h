@@ -142,8 +142,8 @@ int ve_create(const ve_lattice* lattice, const ve_cluster* cluster, const ve_ham
  * max_iter sweeps ran), VE_NOT_CONVERGED, VE_ENONFINITE, VE_EINVAL, VE_ECUDA.  Synchronous. */
 int ve_iterate(ve_handle* h, long max_iter, double tol, ve_status* out);
 
-/* Certified lower bound of the current state, all in float64 on the GPU (eigenvalues by
- * Jacobi).  Synchronous.  Errors: VE_EINVAL, VE_ECUDA. */
+/* Certified lower bound of the current state, everything to float64 accuracy on the GPU
+ * (eigenvalues by Jacobi, those of 16 x 16 blocks in fixed point).  Synchronous.  Errors: VE_EINVAL, VE_ECUDA. */
 int ve_bound(ve_handle* h, ve_cert* out);
 
 /* Release everything the handle owns.  NULL-safe. */
@@ -187,7 +187,8 @@ int ve_get_status(ve_handle* h, ve_status* out);
 int ve_profile(ve_handle* h, int enable);
 int ve_profile_read(ve_handle* h, double* ms, long* launches);
 /* Mean Jacobi sweeps per eigensolve over the profiled sweeps: pair projections (*pair) and
- * wavevector projections (*wavevector); 0 if none ran.  Errors: VE_EINVAL, VE_ECUDA. */
+ * wavevector projections (*wavevector); 0 if none ran, and for 64 x 64 blocks in float64, whose
+ * projections take none (of 16 x 16 blocks in float64 the sweeps are float32 ones).  Errors: VE_EINVAL, VE_ECUDA. */
 int ve_profile_sweeps(ve_handle* h, double* pair, double* wavevector);
 /* How many eigensolves of the profiled sweeps ended with the first-order (Daleckii-Krein)
  * reconstruction instead of a converged Jacobi sweep -- the early stop of the projections of

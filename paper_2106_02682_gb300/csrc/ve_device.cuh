@@ -339,7 +339,7 @@ __device__ __forceinline__ void unit_phase<df64>(df64 br, df64 bi, df64& mag, df
 // the exact stopping rule -- provided also ||E||_F <= d / 4, so that no eigenvalue can reach
 // zero.  float64 takes the sharper form of the same bound: f is exact on either sign's block, so R
 // vanishes with B, the part of E between diagonal entries of opposite sign, and ||R||_F <= c ||B||_F
-// ||E||_F / d (c <= 0.19, tests/test_fx16.py): the sweeps stop once ||B||_F ||E||_F <= n u ||A||_F d.
+// ||E||_F / d (c <= 0.25, tests/test_fx16.py): the sweeps stop once ||B||_F ||E||_F <= n u ||A||_F d.
 // `off` and `nrm` are the squared Frobenius norms of E and A; the test is uniform over the group.
 template <typename T, int n, int LD, int NT>
 __device__ bool dk_stop(const T* A, const T* Ai, T off, T nrm, T* red, int tid) {

@@ -309,7 +309,7 @@ struct Off {
   __device__ __forceinline__ float nrm2() const { return dg + off; }
   // First-order rule.  With f = max(., 0) linear on either side of zero, f(A) = f(Lambda) + L o E +
   // R where R needs the two signs to mix: R vanishes with B, and ||R|| <= c ||B|| ||E|| / d while
-  // ||E|| <= d / 4 (c <= 0.19 over random and clustered spectra, tests/test_fx16.py).  So E between
+  // ||E|| <= d / 4 (c <= 0.25 over random and clustered spectra, tests/test_fx16.py).  So E between
   // eigenvalues of one sign need not be rotated away, and ||B|| ||E|| <= n u ||A|| d / margin stops
   // as accurately as the exact rule (n u: jacobi_sym).
   __device__ __forceinline__ bool first_order(float margin) const {
@@ -850,8 +850,9 @@ __device__ Result project(Frag& ar, Frag& ai, int& ea, long long* v, bool warm, 
   return kProduct;
 }
 
-// A lower bound on the smallest eigenvalue of C (as in project) by one warp: the smallest diagonal
-// entry of A = V^H C V less ||E||_F (Weyl), whether or not the cycle converged.  `sm` holds Smem and
+// A lower bound, up to rounding, on the smallest eigenvalue of C (as in project) by one warp: the smallest
+// diagonal entry of A = V^H C V less ||E||_F (Weyl), whether or not the cycle converged.  Rounding, which
+// nothing is taken off for: 2^-54 of the largest entry in every entry of C, and both products.  `sm` holds Smem and
 // Smem::vectors bytes after it.
 template <bool CPLX>
 __device__ double lowest(Frag& ar, Frag& ai, int ea, unsigned char* sm, int lane) {

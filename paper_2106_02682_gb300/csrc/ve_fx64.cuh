@@ -4,7 +4,7 @@
 // ve_fxsign.cu).
 //
 // Why the sign and not eigenvectors, as at 16 x 16: a float32 Jacobi sweep of a 64 x 64 matrix is 63
-// rounds of CTA barriers, so the eigensolve would cost more than the 39 products of the iteration,
+// rounds of CTA barriers, so the eigensolve would cost more than the 38 products of the projection,
 // which need no starting vectors and no store either.
 //
 // Ten warps own the ten 16 x 16 blocks on and above the diagonal (the others are their conjugate

@@ -5,7 +5,7 @@
 //
 // Why.  The cyclic Jacobi it replaces is a chain of n - 1 dependent round launches a sweep (7.3 us
 // each at n = 512, 6.8 sweeps warm: 27 ms of a 28 ms sweep), and its work is float64.  Here a
-// projection is 39 products, each one launch that fills the chip.
+// projection is 38 products (of one of them all blocks), each one launch that fills the chip.
 //
 // P Y P and not P Y = (Y + sign(Y) Y) / 2, which takes two products less: an error d of the sign leaves
 // d mu of a negative eigenvalue -mu in the latter, and Y has them up to hundreds of times ||X|| (eps G has

@@ -7,7 +7,7 @@
 //   k5_pair    one thread group per pair: H'_ij (Eq. (effHam)), the closed-form rho_ij
 //              (Eq. (rhoijUpdate)), rho~_ij = Pi(rho_ij - Lambda_ij / mu) by the projections of
 //              the Algorithm-6 pair pass (Eq. (rhoijTildeUpdate)): fixed point for D = 16 and 64,
-//              warm-started Jacobi for D = 4 and 256, the Lambda update,
+//              warm-started Jacobi for D = 4, the Lambda update,
 //              A1 rho, A2 rho, and the off-diagonal blocks of Y = X - eps G (G_ij and G_ji =
 //              G_ij^T, Sec. 2.2);
 //   k5_rho     one CTA per cluster: Eq. (rhoiUpdate) over the pairs on either side with the

@@ -121,7 +121,7 @@ size_t bound_ws_bytes(int D);
 
 // D in {4, 16, 64, 256}; arith is an Arith.
 cudaError_t launch_pair(const PairArgs& a, int arith, cudaStream_t s);
-// rho_0 update: two launches (chunk sums over delta, then one CTA), fixed reduction order.
+// rho_0 update: one launch (chunk sums over delta, the last CTA adds them), fixed reduction order.
 cudaError_t launch_rho0(const SmallArgs& a, cudaStream_t s);
 cudaError_t launch_dual_status(const SmallArgs& a, cudaStream_t s);
 
