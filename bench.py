@@ -30,6 +30,7 @@ METRIC = "time-to-certified-bound (residual 1e-6) & ADMM iter/s, warm vs plain, 
 UNIT = "iter/s"
 FP64_PEAK_TFLOPS = 1.25        # nominal GB300 FP64 (152 SMs x 2 FP64 FMA/clk x 2.07 GHz x 2)
 FP32_PEAK_TFLOPS = 80.5        # 152 SMs x 128 FP32 lanes x 2 flop x 2.07 GHz
+ISSUE_PEAK_GINST = 1258.6      # 152 SMs x 4 schedulers x 2.07 GHz, warp instructions
 L2_FLUSH_BYTES = 512 << 20     # > 129 MB L2
 
 
@@ -127,7 +128,7 @@ def stage_work(N, D, npass, ncanon):
 
 # The translation units the Algorithm-6 kernels of the ncu records are compiled from.
 KERNEL_SOURCES = ("ve_bound.cu", "ve_df64.cuh", "ve_device.cuh", "ve_fft.cu", "ve_fx16.cuh",
-                  "ve_sweep.cu")
+                  "ve_fx64.cuh", "ve_fxstep.cuh", "ve_sweep.cu")
 
 
 def source_digest(files=KERNEL_SOURCES):
@@ -328,7 +329,18 @@ def run_ours(args):
         dom = max(prof, key=lambda s: prof[s][0])
         ms_launch = prof[dom][0] / max(1, prof[dom][1])
         wk = work.get(dom, {"flops": 0, "bytes": 0})
-        if dom in ("pair", "xproj"):
+        rec = ncu_record(dom, args.workload, args.precision)
+        if dom in ("pair", "xproj") and D in (16, 64) and prec != 1:
+            # fixed point on the tensor cores: neither float64 nor a memory rate bounds it, but the issue
+            # of its integer, float32 and MMA instructions (counted by ncu on the same sources)
+            inst = rec.get("warp_instructions") if rec else None
+            achieved = inst / (ms_launch * 1e-3) / 1e9 if inst else None
+            roof = {"bound": "issue", "achieved": achieved, "peak": ISSUE_PEAK_GINST,
+                    "unit": "G warp instructions/s",
+                    "frac": achieved / ISSUE_PEAK_GINST if inst else None,
+                    "peak_source": "152 SMs x 4 schedulers x 2.07 GHz",
+                    "nominal_tflops": wk["flops"] / (ms_launch * 1e-3) / 1e12}
+        elif dom in ("pair", "xproj"):
             peak = FP64_PEAK_TFLOPS if prec == 0 else FP32_PEAK_TFLOPS
             achieved = wk["flops"] / (ms_launch * 1e-3) / 1e12
             roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
@@ -355,7 +367,6 @@ def run_ours(args):
                             "FP32 SIMT rate. Per-kernel bounds: profiles/"
                             "launches_tfim1d_L4_N1024_mixed.md")
         roof["ms_per_launch"] = ms_launch
-        rec = ncu_record(dom, args.workload, args.precision)
         roof["traffic"] = rec.get("dram_bytes_per_launch") if rec else None
         if rec and "pipe_busy_while_resident" in rec:
             # the achieved fraction counts nominal flops only; the pipe counter shows how busy

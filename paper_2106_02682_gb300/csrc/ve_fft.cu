@@ -219,6 +219,68 @@ __global__ void __launch_bounds__(256) k_fft_pow2(const PassIo<R> io, const FftP
   }
 }
 
+// The same transform with four points a thread and two stages between exchanges, the same arithmetic in
+// every butterfly (and so the same bits): twice the warps with half the instructions each, for passes
+// whose grid leaves schedulers idle (a float64 instruction of a lone warp takes four times its share of
+// the pipe).  Measured, a transform, k_fft_pow2 and here, us: D = 4, float64, 256 clusters 18.4 and 15.3,
+// 1024 clusters 21.5 and 16.3, 4096 clusters 22.5 and 19.2; float32 17.2 and 12.3, 17.4 and 15.3, 16.3 and
+// 14.7; D = 16, float64, 256 clusters 19.4 and 15.3, 1024 clusters 22.2 and 20.4.  Above the line it loses
+// (D = 64, 64 clusters, 10.4 and 12.2).
+template <typename R, int L>
+__global__ void __launch_bounds__(512) k_fft_quad(const PassIo<R> io, const FftPass ps, const int EC) {
+  using V = typename C2<R>::type;
+  constexpr int n = 1 << L;
+  extern __shared__ __align__(16) unsigned char sraw[];
+  V* sbuf = reinterpret_cast<V*>(sraw);
+  const int la = blockIdx.x / ps.B, lb = blockIdx.x % ps.B;
+  const int e = threadIdx.x % EC, g = threadIdx.x / EC;
+  const int ee = blockIdx.y * EC + e;
+  const bool live = ee < io.E;
+  const double2* Wn = io.tw + ps.w_off;  // exp(-2 pi i t / n)
+  // stage st on positions i0 and i0 + 2^st of the bit-reversed order (as in k_fft_pow2: the twiddles 1
+  // and -i of the first three stages cost no multiplication)
+  auto stage = [&](int st, int i0, V& u, V& b) {
+    const int half = 1 << st, j = i0 & (half - 1);
+    if (st < 3 && (j == 0 || 2 * j == half)) {
+      const V t = j == 0 ? b : C2<R>::make(flip(b.y, io.inv), flip(b.x, ~io.inv));
+      const V a = u;
+      u = C2<R>::make(a.x + t.x, a.y + t.y);
+      b = C2<R>::make(a.x - t.x, a.y - t.y);
+    } else {
+      butterfly(io.twiddle(Wn[j * (n / (2 * half))]), u, b);
+    }
+  };
+  V x[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+    x[r] = live ? io.load(ps, la, lb, bitrev(4 * g + r, L), ee) : C2<R>::make(R(0), R(0));
+#pragma unroll
+  for (int st = 0; st < L; st += 2) {
+    // the thread's positions: q + r 2^st; in the last stage of an odd L the pairs (q, q + n / 2) twice
+    const bool pairs = st + 1 == L;
+    int pos[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      pos[r] = pairs ? g + (r >> 1) * (n / 4) + (r & 1) * (n / 2) : ((g >> st) << (st + 2)) + (g & ((1 << st) - 1)) + (r << st);
+    if (st > 0) {
+      __syncthreads();
+#pragma unroll
+      for (int r = 0; r < 4; ++r) x[r] = sbuf[pos[r] * EC + e];
+    }
+    stage(st, pos[0], x[0], x[1]);
+    stage(st, pos[2], x[2], x[3]);
+    if (!pairs) {
+      stage(st + 1, pos[0], x[0], x[2]);
+      stage(st + 1, pos[1], x[1], x[3]);
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      if (st + 2 < L) sbuf[pos[r] * EC + e] = x[r];  // read by this thread alone before the barrier
+      else if (live) io.store(ps, la, lb, pos[r], ee, x[r]);
+    }
+  }
+}
+
 // Any n <= 64 in float32: the direct sum in shared memory, with the n twiddles there as well (a
 // float64 table entry rounded at every use would cost two conversions at the float64 rate a term).
 __global__ void __launch_bounds__(FFT_THREADS) k_fft_direct(const PassIo<float> io, const FftPass ps, const int EC) {
@@ -926,6 +988,15 @@ cudaError_t run_pass_t(const FftPlan& p, const FftPass& ps, int dir, const doubl
   const dim3 grid((unsigned)lines, (unsigned)((p.E + ec - 1) / ec));
   const size_t smem = sizeof(V) * ps.n * ec;  // at most 32 KB (33 with the direct sum's twiddles)
   const int threads = ps.n > 8 ? ec * (ps.n / 8) : ec;
+  // fewer warps than schedulers (4 x 152; half as many at n = 64, where it has one exchange more): four
+  // points a thread instead of eight
+  const long warps = (long)grid.x * grid.y * ((threads + 31) / 32);
+  if (pow2 && ps.n >= 16 && (ps.n == 64 ? 2 * warps : warps) < 4L * big_grid()) {
+    if (ps.n == 16) k_fft_quad<R, 4><<<grid, ec * 4, smem, s>>>(io, ps, ec);
+    else if (ps.n == 32) k_fft_quad<R, 5><<<grid, ec * 8, smem, s>>>(io, ps, ec);
+    else k_fft_quad<R, 6><<<grid, ec * 16, smem, s>>>(io, ps, ec);
+    return cudaGetLastError();
+  }
   switch (pow2 ? ps.n : 0) {
     case 2: k_fft_pow2<R, 1><<<grid, threads, 0, s>>>(io, ps, ec); break;
     case 4: k_fft_pow2<R, 2><<<grid, threads, 0, s>>>(io, ps, ec); break;
