@@ -373,7 +373,8 @@ def run_ours(args):
             # the unit the kernel is bound by actually is (ncu, same sources)
             roof["ncu_pipe_busy"] = {"pipe": rec["pipe"], "frac": rec["pipe_busy_while_resident"]}
         roof["algorithmic_per_launch"] = wk
-        stages = {s: {"ms_per_launch": prof[s][0] / max(1, prof[s][1]), "launches": prof[s][1],
+        # (a stage without launches holds the gaps between its two events alone)
+        stages = {s: {"ms_per_launch": prof[s][0] / prof[s][1] if prof[s][1] else 0.0, "launches": prof[s][1],
                       "share": prof[s][0] / max(1e-12, sum(v[0] for v in prof.values()))}
                   for s in prof}
         # kernels of one sweep (the captured graph holds the same kernel nodes) x timed sweeps

@@ -707,9 +707,9 @@ __device__ __forceinline__ bool unpack16(const double2* z1, const double2* z2, f
 // of the two and accurate to float64): one warp per canonical wavevector, in the fixed-point form of
 // ve_fx16.cuh.  The block is unpacked (unpack16) and packed back in registers.
 // Without a store the eigenvectors stay in shared memory.
-// Measured (4096 clusters, 2049 blocks): 149 us; 1000 us as float64 Jacobi sweeps (float64 pipe 85 %
-// busy).  Bound by issue: 26k integer, MMA and float32 instructions a block at 42 % of the issue slots
-// (14 warps an SM).
+// Measured (4096 clusters, 2049 blocks): 147 us; 1000 us as float64 Jacobi sweeps (float64 pipe 85 %
+// busy).  Bound by issue: 27k integer, MMA and float32 instructions a block at 41 % of the issue slots
+// (12 warps an SM).
 __global__ void __launch_bounds__(32, 16)
     k_xproj16(double2* spec, const int* __restrict__ canon, const int ncanon, const FftPlan p, const double invN,
               long long* vstore, const int warm, unsigned long long* stats) {
@@ -799,7 +799,7 @@ __global__ void __launch_bounds__(32, 16)
 // projection by the sign iteration of ve_fx64.cuh (no eigenvectors, so no store).  Unpacked entries
 // are recomputed where the iteration needs them; the result passes through shared memory, where an
 // entry meets the one it shares a packed sequence with.
-// Measured (86 blocks of the 170-cluster chain, one wave): 701 us; 6243 us as float64 Jacobi sweeps.
+// Measured (86 blocks of the 170-cluster chain, one wave): 719 us; 6243 us as float64 Jacobi sweeps.
 __global__ void __launch_bounds__(fx64::kThreads, 1)
     k_xproj64(double2* spec, const int* __restrict__ canon, const int ncanon, const FftPlan p, const double invN,
               unsigned long long* stats) {

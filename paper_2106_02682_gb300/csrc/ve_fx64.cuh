@@ -10,8 +10,9 @@
 // Ten warps own the ten 16 x 16 blocks on and above the diagonal (the others are their conjugate
 // transposes), so a product is 4 x 52 MMAs a warp (complex: 4 x 208).  The iterate and the second
 // operand live in shared memory as digit fragments (96 KB each when complex); a block of X^2 stays
-// in its warp's registers for the polynomial.  The tensor pipe bounds it (2.7 SM cycles an MMA):
-// ~13 us a complex product, ~3.5 us a real one.
+// in its warp's registers for the polynomial.  ~18 us a complex product, ~6 us a real one:
+// the tensor pipe is 48 and 30 % busy, the rest is ten warps waiting for their MMAs and at the barriers of
+// the dependent steps.
 #pragma once
 
 #include "ve_fxstep.cuh"
