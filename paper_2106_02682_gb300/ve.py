@@ -616,7 +616,7 @@ def ve_general_profile_read(h):
 
 
 def ve_general_profile_rounds(h):
-    """(ms of the profiled Jacobi sweeps, round launches in them, X steps ended first-order)."""
+    """(ms of the profiled X steps, the launches they held, 0)."""
     ms, r, fo = c_double(), c_long(), c_long()
     _check(_lib.ve_general_profile_rounds(c_void_p(h), ctypes.byref(ms), ctypes.byref(r),
                                           ctypes.byref(fo)), "ve_general_profile_rounds")
